@@ -112,10 +112,12 @@ typedef enum {
   QS_METHOD_BLOCKS_BF16 = 3, /* three BF16 parts, 6 products (~6e-7 relative over 100 blocks) */
   /* the default (also when opts is NULL): for complex64 states with n >= 12
    * the circuit is cut into 5-qubit blocks; a block with more than half of its
-   * 1024 entries nonzero is a dense contraction and runs as a BF16-split GEMM on
-   * the tensor cores, and each maximal run of sparser blocks (diagonal or nearly
-   * diagonal stretches, permutations) is replayed gate by gate through the tile
-   * passes.  With only one or two dense blocks, the whole circuit runs on tile
+   * 1024 entries nonzero is a dense contraction and its gates run as BF16-split
+   * GEMMs on the tensor cores (planned again as chains of up to three 5-qubit blocks
+   * per sweep; one block per sweep when an explicit matrix is not unitary), and each
+   * maximal run of sparser blocks (diagonal or nearly diagonal stretches,
+   * permutations) is replayed gate by gate through the tile passes (runs of up to
+   * four sparse blocks stay with their neighbours in mostly dense circuits).  With only one or two dense blocks, the whole circuit runs on tile
    * passes when that takes no more tile passes and remaps than the sparse runs
    * alone (the blocks' sweeps are saved).  Other states use QS_METHOD_TILED.
    * Synchronous like the block methods. */

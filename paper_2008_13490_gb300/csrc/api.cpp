@@ -11,6 +11,7 @@
 
 #include "abi_guard.h"
 #include "auto_plan.h"
+#include "chain.h"
 #include "fuse_merge.h"
 #include "host_par.h"
 #include "internal.h"
@@ -771,6 +772,73 @@ qs_status run_block_list(State* st, const std::vector<Block>& blocks, int mode, 
   return QS_OK;
 }
 
+// Chains of 5-qubit blocks (chain_tc.cu): up to kChainMax blocks per sweep.
+qs_status run_chains(State* st, const qs_gate* gates, size_t ngates, qs_stats* stats, KernelTimer& tm) {
+  std::vector<ChainPlan> plan;
+  plan_chains(gates, ngates, st->n, plan);
+  std::vector<ChainPass> passes(plan.size());
+  std::vector<const Block*> blocks;
+  std::vector<size_t> first;   // of each pass, into blocks
+  for (size_t i = 0; i < plan.size(); ++i) {
+    uint64_t mask[kChainMax] = {};
+    first.push_back(blocks.size());
+    for (size_t b = 0; b < plan[i].blocks.size(); ++b) {
+      for (int q : plan[i].blocks[b].q) mask[b] |= 1ull << q;
+      blocks.push_back(&plan[i].blocks[b]);
+    }
+    if (!chain_pass_desc(st->n, plan[i].tile, mask, (int)plan[i].blocks.size(), passes[i])) {
+      set_error("block chain: invalid tile");
+      return QS_EUNSUPPORTED;
+    }
+  }
+  std::vector<unsigned char> blob(16 + blocks.size() * (size_t)kChainB, 0);   // status word, B operands
+  parallel_for(blocks.size(), 8, [&](size_t i) { chain_b_operand(blocks[i]->U.data(), blob.data() + 16 + i * kChainB); });
+  qs_status s = upload(st, blob);
+  if (s != QS_OK) return s;
+  unsigned char* dev = (unsigned char*)st->opbuf;
+  int* status_dev = (int*)dev;
+  for (size_t i = 0; i < passes.size(); ++i) {
+    tm.before(4);
+    s = launch_chain_pass(st, passes[i], dev + 16 + first[i] * kChainB, status_dev);
+    tm.after();
+    if (s != QS_OK) return s;
+  }
+  int status = 0;
+  QS_CUDA(cudaMemcpyAsync(&status, status_dev, sizeof(int), cudaMemcpyDeviceToHost, st->stream));
+  QS_CUDA(cudaStreamSynchronize(st->stream));
+  if (status != 0) {
+    set_error(status == QS_ETIMEOUT ? "block chain kernel: bounded wait gave up"
+                                    : "block chain kernel: the tile slots do not fit shared memory");
+    return (qs_status)status;
+  }
+  if (stats) {
+    stats->ops_fused += (int64_t)blocks.size();
+    stats->passes += (int64_t)passes.size();
+    stats->launches += (int64_t)passes.size();
+    stats->flops += 256.0 * std::ldexp(1.0, st->n) * (double)blocks.size();
+    stats->upload_bytes += (int64_t)blob.size();
+  }
+  return QS_OK;
+}
+
+// Every explicit matrix is unitary within 1e-12 (the named gates are by definition): the
+// blocks of a chain then keep each row's norm, which its kernel relies on.
+bool gates_unitary(const qs_gate* gates, size_t ngates) {
+  for (size_t i = 0; i < ngates; ++i) {
+    if (gates[i].kind != QS_MAT1 && gates[i].kind != QS_MAT2) continue;
+    cd m[16];
+    int dim = 0;
+    gate_matrix(gates[i], m, &dim);
+    for (int a = 0; a < dim; ++a)
+      for (int b = a; b < dim; ++b) {
+        cd v = a == b ? cd(-1.0) : cd(0.0);
+        for (int k = 0; k < dim; ++k) v += std::conj(m[k * dim + a]) * m[k * dim + b];
+        if (!(std::abs(v) <= 1e-12)) return false;
+      }
+  }
+  return true;
+}
+
 qs_status run_blocks(State* st, const qs_gate* gates, size_t ngates, int mode, qs_stats* stats,
                      KernelTimer& tm) {
   std::vector<Block> blocks;
@@ -780,7 +848,9 @@ qs_status run_blocks(State* st, const qs_gate* gates, size_t ngates, int mode, q
 
 // QS_METHOD_AUTO (complex64, n >= 12): the circuit is cut into 5-qubit blocks;
 // a dense block (more than half of its 1024 entries nonzero) is a real
-// contraction and goes to the tensor cores, and every maximal run of sparse
+// contraction and goes to the tensor cores (the gates of a run of dense blocks planned
+// again as chains of blocks, one block per sweep if a gate is not unitary), and every
+// maximal run of sparse
 // blocks (diagonal or nearly diagonal stretches such as the QFT's controlled
 // phases) goes back to its gates, which the tile planner fuses into shared-memory
 // passes of 12 qubits.  Both kinds of segment start and end in the canonical
@@ -811,13 +881,22 @@ qs_status run_auto(State* st, const qs_gate* gates, size_t ngates, qs_stats* sta
       return s;
     }
   }
+  const bool chains = gates_unitary(gates, ngates);
+  std::vector<char> is_dense(blocks.size());
+  for (size_t k = 0; k < blocks.size(); ++k) is_dense[k] = block_nonzeros(blocks[k]) > 512;
+  if (chains) auto_short_runs(is_dense);
   size_t i = 0;
   qs_status s = QS_OK;
   while (i < blocks.size() && s == QS_OK) {
-    const bool dense = block_nonzeros(blocks[i]) > 512;
+    const bool dense = is_dense[i];
     size_t j = i;
-    while (j < blocks.size() && (block_nonzeros(blocks[j]) > 512) == dense) ++j;
-    if (dense) {
+    while (j < blocks.size() && (bool)is_dense[j] == dense) ++j;
+    if (dense && chains) {
+      std::vector<qs_gate> seg;
+      for (size_t k = i; k < j; ++k)
+        for (size_t gi : blocks[k].gate_idx) seg.push_back(gates[gi]);
+      s = run_chains(st, seg.data(), seg.size(), stats, tm);
+    } else if (dense) {
       std::vector<Block> seg(std::make_move_iterator(blocks.begin() + (long)i),
                              std::make_move_iterator(blocks.begin() + (long)j));
       s = run_block_list(st, seg, 1, stats, tm);

@@ -16,4 +16,9 @@ namespace qs {
 bool auto_all_tiles(const qs_gate* gates, size_t ngates, int n, const std::vector<Block>& blocks,
                     std::vector<FOp>* fops, std::vector<int>* vmap);
 
+// A run of at most 4 sparse blocks beside dense ones costs a chain pass or two and a tile
+// pass as much or more, so in a circuit of mostly dense blocks (more than 3 for each block of
+// such runs) it stays with its neighbours: marks its blocks dense.
+void auto_short_runs(std::vector<char>& dense);
+
 }  // namespace qs

@@ -144,7 +144,8 @@ struct MaskSet {
   }
 };
 
-// U of block b: the product of its gates, in circuit order
+}  // namespace
+
 void block_product(const qs_gate* gates, Block& b) {
   b.U.assign(32 * 32, cd(0));
   for (int i = 0; i < 32; ++i) b.U[i * 32 + i] = 1.0;
@@ -162,7 +163,20 @@ void block_product(const qs_gate* gates, Block& b) {
   }
 }
 
-}  // namespace
+uint16_t bf16_round_host(float x) {
+  uint32_t u;
+  std::memcpy(&u, &x, 4);
+  const uint32_t lsb = (u >> 16) & 1u;
+  u += 0x7fffu + lsb;   // round to nearest even
+  return (uint16_t)(u >> 16);
+}
+
+float bf16_to_float(uint16_t h) {
+  uint32_t u = (uint32_t)h << 16;
+  float f;
+  std::memcpy(&f, &u, 4);
+  return f;
+}
 
 // Each block takes, among candidate qubit sets, the one that absorbs the most
 // remaining gates (ties: the first candidate): the sets grown from each of the
@@ -256,6 +270,24 @@ bool auto_all_tiles(const qs_gate* gates, size_t ngates, int n, const std::vecto
   int all_passes = 0, all_remaps = 0;   // the whole circuit (its ops stay in *fops)
   count(std::vector<qs_gate>(gates, gates + ngates), &all_passes, &all_remaps);
   return all_passes <= seg_passes && all_remaps <= seg_remaps;
+}
+
+void auto_short_runs(std::vector<char>& dense) {
+  constexpr size_t kShort = 4;
+  size_t n_dense = 0, n_short = 0;
+  std::vector<std::pair<size_t, size_t>> runs;
+  for (size_t i = 0; i < dense.size();) {
+    size_t j = i;
+    while (j < dense.size() && dense[j] == dense[i]) ++j;
+    if (dense[i]) n_dense += j - i;
+    else if (j - i <= kShort) {
+      n_short += j - i;
+      runs.push_back({i, j});
+    }
+    i = j;
+  }
+  if (n_dense <= 3 * n_short) return;
+  for (const auto& r : runs) std::fill(dense.begin() + (long)r.first, dense.begin() + (long)r.second, (char)1);
 }
 
 int block_nonzeros(const Block& b) {

@@ -247,6 +247,11 @@ struct BlockPass {
   uint8_t stage_f[8];
   int32_t n_copy, g_lo, g_len, g0;
 };
+// U of block b: the product of its gates, in circuit order
+void block_product(const qs_gate* gates, Block& b);
+// FP32 to BF16, nearest even, and back
+uint16_t bf16_round_host(float x);
+float bf16_to_float(uint16_t h);
 void block_pass_desc(int n, const int* bpos, BlockPass& P);
 bool block_pass_runs_contiguous(const BlockPass& P);
 // U^dagger U = I within 1e-10 (32x32, row-major)
