@@ -75,18 +75,17 @@ qs_status ensure_opbuf(State* st, size_t bytes) {
   return QS_OK;
 }
 
-// staging of op descriptors: host (pinned) -> device in one copy
-qs_status upload(State* st, const std::vector<unsigned char>& blob) {
-  if (blob.empty()) return QS_OK;
-  qs_status s = ensure_opbuf(st, blob.size());
+// device buffer and pinned staging of at least `bytes`, the staging free to be written
+qs_status reserve_upload(State* st, size_t bytes) {
+  qs_status s = ensure_opbuf(st, bytes);
   if (s != QS_OK) return s;
-  if (st->hostbuf_bytes < blob.size()) {
+  if (st->hostbuf_bytes < bytes) {
     if (st->hostbuf) {
       QS_CUDA(cudaEventSynchronize(st->upload_done));
       cudaFreeHost(st->hostbuf);
     }
     size_t want = 64 * 1024;
-    while (want < blob.size()) want *= 2;
+    while (want < bytes) want *= 2;
     if (cudaMallocHost(&st->hostbuf, want) != cudaSuccess) {
       cudaGetLastError();
       st->hostbuf = nullptr;
@@ -98,9 +97,32 @@ qs_status upload(State* st, const std::vector<unsigned char>& blob) {
   } else {
     QS_CUDA(cudaEventSynchronize(st->upload_done));   // previous copy has read the buffer
   }
+  return QS_OK;
+}
+
+// staging of op descriptors: host (pinned) -> device in one copy
+qs_status upload(State* st, const std::vector<unsigned char>& blob) {
+  if (blob.empty()) return QS_OK;
+  const qs_status s = reserve_upload(st, blob.size());
+  if (s != QS_OK) return s;
   std::memcpy(st->hostbuf, blob.data(), blob.size());
   QS_CUDA(cudaMemcpyAsync(st->opbuf, st->hostbuf, blob.size(), cudaMemcpyHostToDevice, st->stream));
   QS_CUDA(cudaEventRecord(st->upload_done, st->stream));
+  return QS_OK;
+}
+
+// The same for operands that the caller writes into the pinned buffer itself: upload_begin
+// waits for the buffer and hands it out; upload_part queues the copy of [from, to), the last
+// part noted as upload's.
+qs_status upload_begin(State* st, size_t bytes, unsigned char** host) {
+  const qs_status s = reserve_upload(st, bytes);
+  if (s == QS_OK) *host = (unsigned char*)st->hostbuf;
+  return s;
+}
+qs_status upload_part(State* st, size_t from, size_t to, bool last) {
+  QS_CUDA(cudaMemcpyAsync((char*)st->opbuf + from, (char*)st->hostbuf + from, to - from, cudaMemcpyHostToDevice,
+                          st->stream));
+  if (last) QS_CUDA(cudaEventRecord(st->upload_done, st->stream));
   return QS_OK;
 }
 
@@ -772,10 +794,11 @@ qs_status run_block_list(State* st, const std::vector<Block>& blocks, int mode, 
   return QS_OK;
 }
 
-// Chains of 5-qubit blocks (chain_tc.cu): up to kChainMax blocks per sweep.
-qs_status run_chains(State* st, const qs_gate* gates, size_t ngates, qs_stats* stats, KernelTimer& tm) {
-  std::vector<ChainPlan> plan;
-  plan_chains(gates, ngates, st->n, plan);
+// Chains of 5-qubit blocks (chain_tc.cu): up to kChainMax blocks per sweep.  The plan's blocks
+// are multiplied out here, a first part of the passes and then the rest, so that the device
+// starts on the first while the host works on the others (their operands go up in two copies).
+qs_status run_chains(State* st, const qs_gate* gates, const std::vector<ChainPlan>& plan, qs_stats* stats,
+                     KernelTimer& tm) {
   std::vector<ChainPass> passes(plan.size());
   std::vector<const Block*> blocks;
   std::vector<size_t> first;   // of each pass, into blocks
@@ -791,20 +814,40 @@ qs_status run_chains(State* st, const qs_gate* gates, size_t ngates, qs_stats* s
       return QS_EUNSUPPORTED;
     }
   }
-  std::vector<unsigned char> blob(16 + blocks.size() * (size_t)kChainB, 0);   // status word, B operands
-  parallel_for(blocks.size(), 8, [&](size_t i) { chain_b_operand(blocks[i]->U.data(), blob.data() + 16 + i * kChainB); });
-  qs_status s = upload(st, blob);
+  first.push_back(blocks.size());
+  const size_t bytes = 16 + blocks.size() * (size_t)kChainB;   // status word, B operands
+  unsigned char* host = nullptr;
+  qs_status s = upload_begin(st, bytes, &host);
   if (s != QS_OK) return s;
+  s = launch_chain_setup();
+  if (s != QS_OK) return s;
+  std::memset(host, 0, 16);
   unsigned char* dev = (unsigned char*)st->opbuf;
-  int* status_dev = (int*)dev;
-  for (size_t i = 0; i < passes.size(); ++i) {
-    tm.before(4);
-    s = launch_chain_pass(st, passes[i], dev + 16 + first[i] * kChainB, status_dev);
-    tm.after();
-    if (s != QS_OK) return s;
+  const size_t part = passes.size() > 8 ? passes.size() / 4 : passes.size();
+  size_t sent = 0;
+  for (size_t p0 = 0; p0 < passes.size() && s == QS_OK;) {
+    const size_t p1 = p0 == 0 ? part : passes.size();
+    parallel_for(first[p1] - first[p0], 4, [&](size_t k) {
+      cd U[32 * 32];   // (nothing is allocated once a pass has been launched)
+      block_matrix(gates, *blocks[first[p0] + k], U);
+      chain_b_operand(U, host + 16 + (first[p0] + k) * kChainB);
+    });
+    const size_t end = 16 + first[p1] * kChainB;
+    s = upload_part(st, sent, end, p1 == passes.size());
+    sent = end;
+    for (size_t i = p0; i < p1 && s == QS_OK; ++i) {
+      tm.before(4);
+      s = launch_chain_pass(st, passes[i], dev + 16 + first[i] * kChainB, (int*)dev);
+      tm.after();
+    }
+    p0 = p1;
+  }
+  if (s != QS_OK) {   // a copy may still be reading the pinned buffer
+    cudaStreamSynchronize(st->stream);
+    return s;
   }
   int status = 0;
-  QS_CUDA(cudaMemcpyAsync(&status, status_dev, sizeof(int), cudaMemcpyDeviceToHost, st->stream));
+  QS_CUDA(cudaMemcpyAsync(&status, dev, sizeof(int), cudaMemcpyDeviceToHost, st->stream));
   QS_CUDA(cudaStreamSynchronize(st->stream));
   if (status != 0) {
     set_error(status == QS_ETIMEOUT ? "block chain kernel: bounded wait gave up"
@@ -816,7 +859,7 @@ qs_status run_chains(State* st, const qs_gate* gates, size_t ngates, qs_stats* s
     stats->passes += (int64_t)passes.size();
     stats->launches += (int64_t)passes.size();
     stats->flops += 256.0 * std::ldexp(1.0, st->n) * (double)blocks.size();
-    stats->upload_bytes += (int64_t)blob.size();
+    stats->upload_bytes += (int64_t)bytes;
   }
   return QS_OK;
 }
@@ -857,6 +900,12 @@ qs_status run_blocks(State* st, const qs_gate* gates, size_t ngates, int mode, q
 // layout, and applying the blocks in order equals the circuit, so the segments
 // compose.
 qs_status run_auto(State* st, const qs_gate* gates, size_t ngates, qs_stats* stats, KernelTimer& tm) {
+  const bool chains = gates_unitary(gates, ngates);
+  std::vector<ChainPlan> plan;
+  if (chains && chains_likely(gates, ngates)) {   // a circuit of dense layers: all of it as chains
+    plan_chains(gates, ngates, st->n, plan, /*products=*/false);
+    if (chains_dense(gates, plan)) return run_chains(st, gates, plan, stats, tm);
+  }
   std::vector<Block> blocks;
   plan_blocks(gates, ngates, st->n, blocks);
   // one or two dense blocks among sparse ones (the QFT's Hadamards among its
@@ -881,7 +930,6 @@ qs_status run_auto(State* st, const qs_gate* gates, size_t ngates, qs_stats* sta
       return s;
     }
   }
-  const bool chains = gates_unitary(gates, ngates);
   std::vector<char> is_dense(blocks.size());
   for (size_t k = 0; k < blocks.size(); ++k) is_dense[k] = block_nonzeros(blocks[k]) > 512;
   if (chains) auto_short_runs(is_dense);
@@ -895,7 +943,8 @@ qs_status run_auto(State* st, const qs_gate* gates, size_t ngates, qs_stats* sta
       std::vector<qs_gate> seg;
       for (size_t k = i; k < j; ++k)
         for (size_t gi : blocks[k].gate_idx) seg.push_back(gates[gi]);
-      s = run_chains(st, seg.data(), seg.size(), stats, tm);
+      plan_chains(seg.data(), seg.size(), st->n, plan, /*products=*/false);
+      s = run_chains(st, seg.data(), plan, stats, tm);
     } else if (dense) {
       std::vector<Block> seg(std::make_move_iterator(blocks.begin() + (long)i),
                              std::make_move_iterator(blocks.begin() + (long)j));

@@ -21,8 +21,8 @@ namespace {
 // real arithmetic along a row's 32 columns; every complex product is
 // (x_re y_re - x_im y_im, x_re y_im + x_im y_re) and the sums run in gate-entry
 // order, as the complex-typed expressions would compute them.
-void apply_to_block(std::vector<cd>& Uv, const cd* g, int dim, int ia, int ib) {
-  double* U = reinterpret_cast<double*>(Uv.data());   // row r: 32 (re, im) pairs from U + 64 r
+void apply_to_block(cd* Uc, const cd* g, int dim, int ia, int ib) {
+  double* U = reinterpret_cast<double*>(Uc);   // row r: 32 (re, im) pairs from U + 64 r
   // a diagonal gate scales rows (entries exactly 1 leave them alone)
   bool diag = true;
   for (int o = 0; o < dim; ++o)
@@ -147,8 +147,13 @@ struct MaskSet {
 }  // namespace
 
 void block_product(const qs_gate* gates, Block& b) {
-  b.U.assign(32 * 32, cd(0));
-  for (int i = 0; i < 32; ++i) b.U[i * 32 + i] = 1.0;
+  b.U.resize(32 * 32);
+  block_matrix(gates, b, b.U.data());
+}
+
+void block_matrix(const qs_gate* gates, const Block& b, cd* U) {
+  std::fill(U, U + 32 * 32, cd(0));
+  for (int i = 0; i < 32; ++i) U[i * 32 + i] = 1.0;
   auto local = [&](int q) {
     for (int i = 0; i < 5; ++i)
       if (b.q[i] == q) return i;
@@ -159,23 +164,8 @@ void block_product(const qs_gate* gates, Block& b) {
     cd m[16];
     int dim = 0;
     gate_matrix(g, m, &dim);
-    apply_to_block(b.U, m, dim, local(g.q[0]), dim == 4 ? local(g.q[1]) : -1);
+    apply_to_block(U, m, dim, local(g.q[0]), dim == 4 ? local(g.q[1]) : -1);
   }
-}
-
-uint16_t bf16_round_host(float x) {
-  uint32_t u;
-  std::memcpy(&u, &x, 4);
-  const uint32_t lsb = (u >> 16) & 1u;
-  u += 0x7fffu + lsb;   // round to nearest even
-  return (uint16_t)(u >> 16);
-}
-
-float bf16_to_float(uint16_t h) {
-  uint32_t u = (uint32_t)h << 16;
-  float f;
-  std::memcpy(&f, &u, 4);
-  return f;
 }
 
 // Each block takes, among candidate qubit sets, the one that absorbs the most
@@ -292,7 +282,7 @@ void auto_short_runs(std::vector<char>& dense) {
 
 int block_nonzeros(const Block& b) {
   int nz = 0;
-  for (const cd& u : b.U) nz += std::abs(u) > 0.0 ? 1 : 0;
+  for (const cd& u : b.U) nz += u.real() != 0.0 || u.imag() != 0.0 ? 1 : 0;
   return nz;
 }
 

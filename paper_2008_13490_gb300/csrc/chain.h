@@ -18,8 +18,14 @@ struct ChainPlan {
   uint64_t tile = 0;
   std::vector<Block> blocks;
 };
-// Plans gates[0..ngates) (n >= 12) and forms every block's matrix.
-void plan_chains(const qs_gate* gates, size_t ngates, int n, std::vector<ChainPlan>& out);
+// Plans gates[0..ngates) (n >= 12); products: also forms every block's matrix.
+void plan_chains(const qs_gate* gates, size_t ngates, int n, std::vector<ChainPlan>& out, bool products = true);
+// Whether the default method runs the whole circuit as this plan: at least three of its
+// blocks are dense (more than 512 of 1024 entries nonzero) for each that is not.
+bool chains_dense(const qs_gate* gates, const std::vector<ChainPlan>& plan);
+// Whether enough gates make superpositions (neither diagonal nor a permutation) for that to
+// be worth planning: a dense block holds at least five of them.
+bool chains_likely(const qs_gate* gates, size_t ngates);
 
 // Where the element of row m and column c of a block lies in the 32 KiB tile: byte
 // offset = XOR of row[i] over the bits of m and col[i] over the bits of c.
@@ -49,6 +55,8 @@ constexpr int kChainPart = 96 * 32 * 2;
 constexpr int kChainB = 3 * kChainPart;
 void chain_b_operand(const cd* U, unsigned char* out);
 
+// once per call, before its passes
+qs_status launch_chain_setup();
 qs_status launch_chain_pass(State* st, const ChainPass& P, const void* b_dev, int* status_dev);
 
 }  // namespace qs

@@ -103,7 +103,7 @@ int split_tile(const std::vector<uint64_t>& m, uint64_t T, std::vector<uint64_t>
 // with every window of 8 neighbouring qubits) the kTry that take the most gates are split
 // into blocks, and the one whose blocks take the most is kept.  40 layers of Haar + CZ at
 // 30 qubits: 38 passes of 110 blocks.
-void plan_chains(const qs_gate* gates, size_t ngates, int n, std::vector<ChainPlan>& out) {
+void plan_chains(const qs_gate* gates, size_t ngates, int n, std::vector<ChainPlan>& out, bool products) {
   constexpr size_t kSeeds = 12, kTry = 4;
   const uint64_t low = (1ull << kChainLow) - 1, all = n >= 64 ? ~0ull : (1ull << n) - 1;
   out.clear();
@@ -159,10 +159,78 @@ void plan_chains(const qs_gate* gates, size_t ngates, int n, std::vector<ChainPl
     }
     out.push_back(std::move(p));
   }
+  if (!products) return;
   std::vector<Block*> flat;
   for (ChainPlan& p : out)
     for (Block& b : p.blocks) flat.push_back(&b);
   parallel_for(flat.size(), 8, [&](size_t i) { block_product(gates, *flat[i]); });
+}
+
+namespace {
+
+bool branches(const qs_gate& g) {
+  switch (g.kind) {
+    case QS_H: case QS_PX: case QS_MX: case QS_PY: case QS_MY: case QS_RX: case QS_RY: case QS_U2: case QS_U3:
+    case QS_MAT1: case QS_MAT2:
+      return true;
+    default:
+      return false;
+  }
+}
+bool fixed_branch(const qs_gate& g) {
+  return g.kind == QS_H || g.kind == QS_PX || g.kind == QS_MX || g.kind == QS_PY || g.kind == QS_MY;
+}
+
+// block_nonzeros(b) > 512 without the product where its pattern decides: entry (r, c) can be
+// nonzero only if a path of nonzero gate entries leads there.  A pattern that is sparse is
+// certain; sums that cancel exactly come from the fixed gates (H H = 1), so a block with two
+// of those is multiplied out.
+bool block_dense(const qs_gate* gates, const Block& b) {
+  uint32_t row[32];
+  for (int r = 0; r < 32; ++r) row[r] = 1u << r;
+  int fixed = 0;
+  for (size_t gi : b.gate_idx) {
+    const qs_gate& g = gates[gi];
+    if (!branches(g) && g.kind < QS_CNOT && g.kind != QS_X && g.kind != QS_Y) continue;   // diagonal
+    fixed += fixed_branch(g);
+    cd m[16];
+    int dim = 0, at[2] = {0, 0};
+    gate_matrix(g, m, &dim);
+    for (int k = 0; k < (dim == 4 ? 2 : 1); ++k)
+      for (int i = 0; i < 5; ++i)
+        if (b.q[i] == g.q[k]) at[k] = i;
+    const int hi = 1 << at[0], lo = dim == 4 ? 1 << at[1] : 0;
+    for (int r = 0; r < 32; ++r) {
+      if ((r & hi) || (r & lo)) continue;
+      const int idx[4] = {r, dim == 4 ? r | lo : r | hi, r | hi, r | hi | lo};
+      uint32_t out[4] = {0, 0, 0, 0};
+      for (int i = 0; i < dim; ++i)
+        for (int k = 0; k < dim; ++k)
+          if (m[i * dim + k] != cd(0)) out[i] |= row[idx[k]];
+      for (int i = 0; i < dim; ++i) row[idx[i]] = out[i];
+    }
+  }
+  int nz = 0;
+  for (int r = 0; r < 32; ++r) nz += __builtin_popcount(row[r]);
+  if (nz <= 512 || fixed < 2) return nz > 512;
+  Block c = b;
+  block_product(gates, c);
+  return block_nonzeros(c) > 512;
+}
+
+}  // namespace
+
+bool chains_likely(const qs_gate* gates, size_t ngates) {
+  size_t k = 0;
+  for (size_t i = 0; i < ngates; ++i) k += branches(gates[i]);
+  return 5 * k > ngates;
+}
+
+bool chains_dense(const qs_gate* gates, const std::vector<ChainPlan>& plan) {
+  int dense = 0, sparse = 0;
+  for (const ChainPlan& p : plan)
+    for (const Block& b : p.blocks) ++(block_dense(gates, b) ? dense : sparse);
+  return dense > 0 && dense >= 3 * sparse;
 }
 
 namespace {
@@ -298,15 +366,24 @@ bool chain_pass_desc(int n, uint64_t tile, const uint64_t* blocks, int nblk, Cha
 // outputs in columns 0..31 and 32..63; those with the imaginary parts read rows 0..63.
 // K-major core matrices of 8 rows x 16 bytes, no swizzle.
 void chain_b_operand(const cd* U, unsigned char* out) {
-  for (int row = 0; row < 96; ++row)
-    for (int k = 0; k < 32; ++k) {
-      const cd u = U[(row & 31) * 32 + k];
-      double r = row < 32 ? -u.imag() : row < 64 ? u.real() : u.imag();
-      const int off = (row >> 3) * 512 + (k >> 3) * 128 + (row & 7) * 16 + (k & 7) * 2;
-      for (int p = 0; p < 3; ++p) {
-        const uint16_t h = bf16_round_host((float)r);
-        r -= (double)bf16_to_float(h);
-        std::memcpy(out + p * kChainPart + off, &h, 2);
+  for (int row = 0; row < 32; ++row)
+    for (int k0 = 0; k0 < 32; k0 += 8) {
+      uint16_t re[3][8], im[3][8], neg[3][8];
+      for (int k = 0; k < 8; ++k) {
+        double a = U[row * 32 + k0 + k].real(), c = U[row * 32 + k0 + k].imag();
+        for (int p = 0; p < 3; ++p) {
+          re[p][k] = bf16_round_host((float)a);
+          im[p][k] = bf16_round_host((float)c);
+          neg[p][k] = im[p][k] ^ 0x8000u;
+          a -= (double)bf16_to_float(re[p][k]);
+          c -= (double)bf16_to_float(im[p][k]);
+        }
+      }
+      unsigned char* at = out + (row >> 3) * 512 + (k0 >> 3) * 128 + (row & 7) * 16;
+      for (int p = 0; p < 3; ++p, at += kChainPart) {
+        std::memcpy(at, neg[p], 16);
+        std::memcpy(at + 4 * 512, re[p], 16);
+        std::memcpy(at + 8 * 512, im[p], 16);
       }
     }
 }

@@ -526,6 +526,11 @@ qs_status chain_tensor_map(const State* st, const ChainPass& P, CUtensorMap* map
 
 }  // namespace
 
+qs_status launch_chain_setup() {
+  QS_CUDA(cudaFuncSetAttribute(chain_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kDynSmem));
+  return QS_OK;
+}
+
 qs_status launch_chain_pass(State* st, const ChainPass& P, const void* b_dev, int* status_dev) {
   CUtensorMap map;
   const qs_status ms = chain_tensor_map(st, P, &map);
@@ -537,7 +542,6 @@ qs_status launch_chain_pass(State* st, const ChainPass& P, const void* b_dev, in
   // one CTA holds all tensor memory of its SM; leave the SMs a server's persistent kernel may hold
   uint64_t grid = (uint64_t)std::max(1, sms - reserved_sms());
   if (grid > ntiles) grid = ntiles;
-  QS_CUDA(cudaFuncSetAttribute(chain_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kDynSmem));
   chain_kernel<<<(unsigned)grid, kThreads, kDynSmem, st->stream>>>(P, map, (const unsigned char*)b_dev, (uint32_t)ntiles,
                                                                status_dev);
   QS_CUDA(cudaGetLastError());

@@ -5,6 +5,7 @@
 #include <stdint.h>
 
 #include <complex>
+#include <cstring>
 #include <string>
 #include <vector>
 
@@ -249,9 +250,21 @@ struct BlockPass {
 };
 // U of block b: the product of its gates, in circuit order
 void block_product(const qs_gate* gates, Block& b);
+// the same into a caller's 32x32 (nothing is allocated; b.U is not touched)
+void block_matrix(const qs_gate* gates, const Block& b, cd* U);
 // FP32 to BF16, nearest even, and back
-uint16_t bf16_round_host(float x);
-float bf16_to_float(uint16_t h);
+inline uint16_t bf16_round_host(float x) {
+  uint32_t u;
+  std::memcpy(&u, &x, 4);
+  u += 0x7fffu + ((u >> 16) & 1u);
+  return (uint16_t)(u >> 16);
+}
+inline float bf16_to_float(uint16_t h) {
+  const uint32_t u = (uint32_t)h << 16;
+  float f;
+  std::memcpy(&f, &u, 4);
+  return f;
+}
 void block_pass_desc(int n, const int* bpos, BlockPass& P);
 bool block_pass_runs_contiguous(const BlockPass& P);
 // U^dagger U = I within 1e-10 (32x32, row-major)
