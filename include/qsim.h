@@ -119,7 +119,10 @@ typedef enum {
    * permutations) is replayed gate by gate through the tile passes (runs of up to
    * four sparse blocks stay with their neighbours in mostly dense circuits).  With only one or two dense blocks, the whole circuit runs on tile
    * passes when that takes no more tile passes and remaps than the sparse runs
-   * alone (the blocks' sweeps are saved).  Other states use QS_METHOD_TILED.
+   * alone (the blocks' sweeps are saved).  complex128 states with n >= 12: circuits of
+   * mostly dense blocks run block by block on the tensor cores too, in exact integer
+   * slices of the FP64 values (one rounding per block and amplitude).  Everything else
+   * uses QS_METHOD_TILED.
    * Synchronous like the block methods. */
   QS_METHOD_AUTO = 4
 } qs_method;

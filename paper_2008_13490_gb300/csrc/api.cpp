@@ -1,4 +1,5 @@
 // C ABI entry points of the state-vector path (see include/qsim.h).
+#include <algorithm>
 #include <cstdarg>
 #include <cstdio>
 #include <complex>
@@ -11,6 +12,7 @@
 
 #include "abi_guard.h"
 #include "auto_plan.h"
+#include "block_f64.h"
 #include "chain.h"
 #include "fuse_merge.h"
 #include "host_par.h"
@@ -889,6 +891,61 @@ qs_status run_blocks(State* st, const qs_gate* gates, size_t ngates, int mode, q
   return run_block_list(st, blocks, mode, stats, tm);
 }
 
+// QS_METHOD_AUTO, complex128, n >= 12: circuits of mostly dense blocks (at least three for each
+// sparse one) run block by block on the tensor cores (block_f64.cu).  QS_EUNSUPPORTED, with
+// nothing launched, for others and for matrices that the integer slices do not take: they run
+// on tile passes.
+qs_status run_f64_blocks(State* st, const qs_gate* gates, size_t ngates, qs_stats* stats, KernelTimer& tm) {
+  if (!chains_likely(gates, ngates)) return QS_EUNSUPPORTED;
+  std::vector<Block> blocks;
+  plan_blocks(gates, ngates, st->n, blocks, /*products=*/false);
+  size_t dense = 0;
+  for (const Block& b : blocks) dense += block_dense(gates, b);
+  if (dense == 0 || dense < 3 * (blocks.size() - dense)) return QS_EUNSUPPORTED;
+  std::vector<F64Pass> passes(blocks.size());
+  for (size_t i = 0; i < blocks.size(); ++i)
+    if (!f64_pass_desc(st->n, blocks[i].q, passes[i])) return QS_EUNSUPPORTED;
+  const size_t bytes = 16 + blocks.size() * (size_t)kF64B;   // status word, B operands
+  unsigned char* host = nullptr;
+  qs_status s = upload_begin(st, bytes, &host);
+  if (s != QS_OK) return s;
+  std::memset(host, 0, 16);
+  std::vector<char> fits(blocks.size());
+  parallel_for(blocks.size(), 2, [&](size_t i) {
+    fits[i] = f64_b_operand(gates, blocks[i], host + 16 + i * kF64B, &passes[i].vs);
+  });
+  if (std::find(fits.begin(), fits.end(), (char)0) != fits.end()) return QS_EUNSUPPORTED;
+  s = launch_f64_setup();
+  if (s != QS_OK) return s;
+  unsigned char* dev = (unsigned char*)st->opbuf;
+  s = upload_part(st, 0, bytes, true);
+  for (size_t i = 0; i < blocks.size() && s == QS_OK; ++i) {
+    tm.before(4);
+    s = launch_f64_pass(st, passes[i], dev + 16 + i * kF64B, (int*)dev);
+    tm.after();
+  }
+  if (s != QS_OK) {
+    cudaStreamSynchronize(st->stream);
+    return s == QS_EUNSUPPORTED ? QS_ECUDA : s;
+  }
+  int status = 0;
+  QS_CUDA(cudaMemcpyAsync(&status, dev, sizeof(int), cudaMemcpyDeviceToHost, st->stream));
+  QS_CUDA(cudaStreamSynchronize(st->stream));
+  if (status != 0) {
+    set_error(status == QS_ETIMEOUT ? "complex128 block kernel: bounded wait gave up"
+                                    : "complex128 block kernel: the tile slots do not fit shared memory");
+    return status == QS_ETIMEOUT ? QS_ETIMEOUT : QS_ECUDA;
+  }
+  if (stats) {
+    stats->ops_fused += (int64_t)blocks.size();
+    stats->passes += (int64_t)blocks.size();
+    stats->launches += (int64_t)blocks.size();
+    stats->flops += 256.0 * std::ldexp(1.0, st->n) * (double)blocks.size();
+    stats->upload_bytes += (int64_t)bytes;
+  }
+  return QS_OK;
+}
+
 // QS_METHOD_AUTO (complex64, n >= 12): the circuit is cut into 5-qubit blocks;
 // a dense block (more than half of its 1024 entries nonzero) is a real
 // contraction and goes to the tensor cores (the gates of a run of dense blocks planned
@@ -1010,6 +1067,7 @@ qs_status apply_gates(State* st, const qs_gate* gates, size_t ngates, int method
   }
   // AUTO: blocks and tile passes where the state allows the blocks, else tiles
   const bool autom = method == QS_METHOD_AUTO && st->prec == QS_C64 && st->n >= kTileBits;
+  const bool auto_f64 = method == QS_METHOD_AUTO && st->prec == QS_C128 && st->n >= kTileBits;
   if (method == QS_METHOD_AUTO && !autom) method = QS_METHOD_TILED;
   const bool blocks = method == QS_METHOD_BLOCKS_TF32 || method == QS_METHOD_BLOCKS_BF16;
   if (blocks && (st->prec != QS_C64 || st->n < kTileBits)) {
@@ -1023,8 +1081,10 @@ qs_status apply_gates(State* st, const qs_gate* gates, size_t ngates, int method
   KernelTimer tm;
   tm.on = (flags & QS_OPT_TIME_KERNELS) != 0;
   tm.stream = st->stream;
-  qs_status s;
-  if (autom) {
+  qs_status s = QS_EUNSUPPORTED;
+  if (auto_f64) s = run_f64_blocks(st, gates, ngates, stats, tm);
+  if (auto_f64 && s != QS_EUNSUPPORTED) {
+  } else if (autom) {
     s = run_auto(st, gates, ngates, stats, tm);
   } else if (blocks) {
     s = run_blocks(st, gates, ngates, method == QS_METHOD_BLOCKS_TF32 ? 0 : 1, stats, tm);

@@ -174,7 +174,7 @@ void block_matrix(const qs_gate* gates, const Block& b, cd* U) {
 // light cones of nearest-neighbour circuits).  On 40 layers of Haar + brickwork
 // CZ at 30 qubits this gives 100 blocks where growing from the first remaining
 // gate alone gives 148.
-void plan_blocks(const qs_gate* gates, size_t ngates, int n, std::vector<Block>& out) {
+void plan_blocks(const qs_gate* gates, size_t ngates, int n, std::vector<Block>& out, bool products) {
   constexpr int kSeeds = 64;
   out.clear();
   std::vector<size_t> remaining(ngates);
@@ -230,6 +230,7 @@ void plan_blocks(const qs_gate* gates, size_t ngates, int n, std::vector<Block>&
     rem_m.resize(w);
   }
   // each block's product of its gates (blocks are independent)
+  if (!products) return;
   parallel_for(out.size(), 8, [&](size_t bi) { block_product(gates, out[bi]); });
 }
 

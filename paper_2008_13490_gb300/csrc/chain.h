@@ -20,6 +20,8 @@ struct ChainPlan {
 };
 // Plans gates[0..ngates) (n >= 12); products: also forms every block's matrix.
 void plan_chains(const qs_gate* gates, size_t ngates, int n, std::vector<ChainPlan>& out, bool products = true);
+// block_nonzeros(b) > 512, mostly from the gates' patterns (b.U is not needed)
+bool block_dense(const qs_gate* gates, const Block& b);
 // Whether the default method runs the whole circuit as this plan: at least three of its
 // blocks are dense (more than 512 of 1024 entries nonzero) for each that is not.
 bool chains_dense(const qs_gate* gates, const std::vector<ChainPlan>& plan);

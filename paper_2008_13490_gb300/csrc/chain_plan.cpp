@@ -181,6 +181,8 @@ bool fixed_branch(const qs_gate& g) {
   return g.kind == QS_H || g.kind == QS_PX || g.kind == QS_MX || g.kind == QS_PY || g.kind == QS_MY;
 }
 
+}  // namespace
+
 // block_nonzeros(b) > 512 without the product where its pattern decides: entry (r, c) can be
 // nonzero only if a path of nonzero gate entries leads there.  A pattern that is sparse is
 // certain; sums that cancel exactly come from the fixed gates (H H = 1), so a block with two
@@ -217,8 +219,6 @@ bool block_dense(const qs_gate* gates, const Block& b) {
   block_product(gates, c);
   return block_nonzeros(c) > 512;
 }
-
-}  // namespace
 
 bool chains_likely(const qs_gate* gates, size_t ngates) {
   size_t k = 0;

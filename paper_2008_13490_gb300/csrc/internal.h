@@ -219,7 +219,7 @@ struct Block {
 // entries of a block with |U_ij| > 0 (dense: more than half of the 1024)
 int block_nonzeros(const Block& b);
 // Greedy frontier fusion of the circuit into 5-qubit blocks (n >= 5).
-void plan_blocks(const qs_gate* gates, size_t ngates, int n, std::vector<Block>& out);
+void plan_blocks(const qs_gate* gates, size_t ngates, int n, std::vector<Block>& out, bool products = true);
 // Tile of a block pass: 12 positions = 5 block qubits + 7 row qubits; the
 // tables map an element's "address-order" index (its 12 tile bits sorted by
 // physical position, split 6 + 6) to its address offset, row m and column c.
