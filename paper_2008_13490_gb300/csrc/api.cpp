@@ -1434,7 +1434,7 @@ qs_status sv_probs(qs_state_t st, void* out, int out_fp64, uint64_t marg_mask, d
     unsigned char* sc = (unsigned char*)st->scratch;
     double* partials = (double*)(sc + kScratchPartials);
     s = launch_probs(st, out, out_fp64, marginal ? marg_mask : 0, partials,
-                     (uint8_t*)(sc + kScratchBits), (double*)(sc + kScratchMarg));
+                     (double*)(sc + kScratchMarg));
     if (s != QS_OK) return s;
     if (norm_out) {
       double* res = (double*)(sc + kScratchResult);

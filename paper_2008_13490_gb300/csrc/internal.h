@@ -60,7 +60,6 @@ constexpr int kReduceBlocks = 1024;               // partial sums written by red
 constexpr size_t kScratchPartials = 0;            // kReduceBlocks doubles
 constexpr size_t kScratchClamps = 8192;           // one 64-bit counter
 constexpr size_t kScratchResult = 8448;           // 16 doubles
-constexpr size_t kScratchBits = 8704;             // 64 bytes of bit positions
 constexpr size_t kScratchMarg = 16384;            // marginal accumulators (doubles)
 constexpr int kScratchMargLog2 = 16;              // largest marginal kept in scratch
 constexpr size_t kScratchBytes = kScratchMarg + (sizeof(double) << kScratchMargLog2);
@@ -314,7 +313,7 @@ qs_status launch_plain_op(State* st, const void* op_dev, int type);
 qs_status launch_small(State* st, const void* ops_dev, int nops);
 qs_status launch_remap(State* st, const RemapDesc& desc);
 qs_status launch_probs(State* st, void* out, int out_fp64, uint64_t mask, double* partials,
-                       uint8_t* bits_dev, double* marg_acc);
+                       double* marg_acc);
 // probabilities of amplitudes [off, off + count) of the state into out (device;
 // float or double), block partial sums of that range into partials
 qs_status launch_probs_range(State* st, uint64_t off, uint64_t count, void* out, int out_fp64,

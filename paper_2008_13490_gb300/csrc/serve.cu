@@ -499,7 +499,7 @@ struct Server {
           double* marg = (double*)(sc + kScratchMarg);
           const bool all = r->k == r->n;   // a mask of all n bits is the plain distribution
           s2 = launch_probs(st, all ? marg : nullptr, 1, all ? 0 : r->mask, (double*)(sc + kScratchPartials),
-                            (uint8_t*)(sc + kScratchBits), marg);
+                            marg);
           if (s2 == QS_OK) {
             cudaError_t e = cudaMemcpyAsync(hbuf, marg, sizeof(double) << r->k, cudaMemcpyDeviceToHost, stream);
             if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
