@@ -1,5 +1,6 @@
 // C ABI entry points of the state-vector path (see include/qsim.h).
 #include <algorithm>
+#include <array>
 #include <cstdarg>
 #include <cstdio>
 #include <complex>
@@ -602,13 +603,163 @@ qs_status run_tiled(State* st, const std::vector<FOp>& fops, const std::vector<i
   return QS_OK;
 }
 
-// The adjoint sweep over gates [g0, g1) fused into tile passes.  The reversed
-// gate list becomes, per gate, one op per parameter carrying its derivative
-// matrix G_p = (dU/dt_p) U^dagger (a term op, not applied) followed by
-// U^dagger; the tile planner splits it into passes (an op keeps its order with
-// the ops that share a qubit), and each pass runs the adjoint pass kernel on
-// psi = st->data and lam, its per-tile terms reduced into dth.  Dense two-qubit
-// U^dagger ops (SWAP, MAT2) run as plain launches on both states.
+// The gates [g0, g1) backwards as the ops of the adjoint sweep (internal.h, FOp::term).  A run of
+// one-qubit gates on a qubit, nothing else on it in between, becomes one op at the place of its last
+// gate: the product W of the gates' U^dagger, and the derivatives of all of its parameters as
+// combinations of the sums of a TermRec.  (G = (dU/dt) U^dagger of a gate before which the product W'
+// is already undone acts as W'^dagger G W' on the states after the run; it is anti-Hermitian as G is.)
+// Runs of diagonal gates alone stay diagonals, which need no place in a tile: per gate one op with G
+// for each parameter and one with U^dagger.  Diagonals without a term then go into the ops before them.
+struct AdjointOps {
+  std::vector<FOp> ops;
+  std::vector<TermRec> recs;   // sum: filled in per pass
+  std::vector<TermPar> pars;
+};
+qs_status adjoint_ops(const qs_gate* gates, size_t g0, size_t g1, int n, AdjointOps& out) {
+  // runs: per gate the run it belongs to; runs that hold a non-diagonal matrix
+  std::vector<int> run(g1 - g0, -1), open(n, -1);
+  std::vector<char> dense;
+  auto zero = [](cd z) { return z.real() == 0.0 && z.imag() == 0.0; };
+  auto derivative = [](const qs_gate& G, int p, const cd* Ud, int dim, cd* M) {   // (dU/dt_p) U^dagger
+    cd dU[16];
+    gate_dmatrix(G, p, dU);
+    for (int r = 0; r < dim; ++r)
+      for (int c = 0; c < dim; ++c) {
+        cd acc = 0;
+        for (int k = 0; k < dim; ++k) acc += dU[r * dim + k] * Ud[k * dim + c];
+        M[r * dim + c] = acc;
+      }
+  };
+  auto dagger = [](const qs_gate& G, cd* Ud, int* dim) {
+    cd U[16];
+    gate_matrix(G, U, dim);
+    for (int r = 0; r < *dim; ++r)
+      for (int c = 0; c < *dim; ++c) Ud[r * *dim + c] = std::conj(U[c * *dim + r]);
+  };
+  for (size_t g = g1; g-- > g0;) {
+    const qs_gate& G = gates[g];
+    cd Ud[16], M[16];
+    int dim = 0;
+    dagger(G, Ud, &dim);
+    if (dim != 2) {
+      open[G.q[0]] = open[G.q[1]] = -1;
+      continue;
+    }
+    int& o = open[G.q[0]];
+    if (o < 0) {
+      o = (int)dense.size();
+      dense.push_back(0);
+    }
+    run[g - g0] = o;
+    bool d = zero(Ud[1]) && zero(Ud[2]);
+    for (int p = 0; p < gate_nparams(G.kind) && d; ++p) {
+      derivative(G, p, Ud, 2, M);
+      d = zero(M[1]) && zero(M[2]);
+    }
+    if (!d) dense[(size_t)o] = 1;
+  }
+  std::vector<qs_gate> bw;
+  std::vector<int> term;                       // per op: its record
+  std::vector<int> run_op(dense.size(), -1);   // the op of a dense run
+  std::vector<std::array<cd, 4>> W(dense.size());
+  std::vector<std::vector<TermPar>> pars;      // per record
+  auto as_gate = [](const qs_gate& G, const cd* m, int dim) {
+    qs_gate x;
+    std::memset(&x, 0, sizeof(x));
+    x.kind = dim == 2 ? QS_MAT1 : QS_MAT2;
+    x.q[0] = G.q[0];
+    x.q[1] = dim == 2 ? 0 : G.q[1];
+    for (int i = 0; i < dim * dim; ++i) {
+      x.m[2 * i] = m[i].real();
+      x.m[2 * i + 1] = m[i].imag();
+    }
+    return x;
+  };
+  auto record = [&](int nsum) {
+    out.recs.push_back(TermRec{0, nsum, 0, 0});
+    pars.emplace_back();
+    return (int)out.recs.size() - 1;
+  };
+  auto mul2 = [](const cd* A, const cd* B, cd* C) {
+    cd r[4] = {A[0] * B[0] + A[1] * B[2], A[0] * B[1] + A[1] * B[3], A[2] * B[0] + A[3] * B[2],
+               A[2] * B[1] + A[3] * B[3]};
+    for (int i = 0; i < 4; ++i) C[i] = r[i];
+  };
+  for (size_t g = g1; g-- > g0;) {
+    const qs_gate& G = gates[g];
+    cd Ud[16], M[16];
+    int dim = 0;
+    dagger(G, Ud, &dim);
+    const int np = gate_nparams(G.kind), r = run[g - g0];
+    if (r < 0 || !dense[(size_t)r]) {
+      for (int p = 0; p < np; ++p) {
+        derivative(G, p, Ud, dim, M);
+        bw.push_back(as_gate(G, M, dim));
+        term.push_back(record(1));
+        pars.back().push_back(TermPar{(int64_t)(3 * g + p), {1.0, 0.0, 0.0, 0.0}});
+      }
+      bw.push_back(as_gate(G, Ud, dim));
+      term.push_back(-1);
+      continue;
+    }
+    cd* w = W[(size_t)r].data();
+    const bool first = run_op[(size_t)r] < 0;
+    if (first) {
+      run_op[(size_t)r] = (int)bw.size();
+      bw.push_back(as_gate(G, Ud, dim));   // the place; its matrix is the run's W, below
+      term.push_back(-1);
+      w[0] = w[3] = 1;
+      w[1] = w[2] = 0;
+    }
+    int& t = term[(size_t)run_op[(size_t)r]];
+    for (int p = 0; p < np; ++p) {
+      if (t < 0) t = record(4);
+      cd Wd[4] = {std::conj(w[0]), std::conj(w[2]), std::conj(w[1]), std::conj(w[3])};
+      derivative(G, p, Ud, 2, M);
+      mul2(Wd, M, M);
+      mul2(M, w, M);
+      pars[(size_t)t].push_back(TermPar{(int64_t)(3 * g + p),
+                                        {-M[0].imag(), -M[3].imag(), 0.5 * (M[1].real() - M[2].real()),
+                                         -0.5 * (M[1].imag() + M[2].imag())}});
+    }
+    mul2(Ud, w, w);
+  }
+  std::vector<int> vmap;
+  build_fused_ops(bw.data(), bw.size(), n, out.ops, vmap, /*fuse=*/false, /*relabel=*/false);
+  if (out.ops.size() != bw.size()) {
+    set_error("adjoint op list changed size");
+    return QS_EUNSUPPORTED;
+  }
+  for (size_t i = 0; i < out.ops.size(); ++i) {
+    out.ops[i].term = term[i];
+    if (term[i] >= 0 && out.recs[(size_t)term[i]].nsum == 1 && out.ops[i].type != F_D) {
+      set_error("derivative matrix of gate %d is not a one-qubit or diagonal op", (int)(pars[(size_t)term[i]][0].slot / 3));
+      return QS_EUNSUPPORTED;
+    }
+  }
+  for (size_t r = 0; r < W.size(); ++r) {
+    if (run_op[r] < 0) continue;
+    FOp& o = out.ops[(size_t)run_op[r]];
+    const int tm = o.term, q = bw[(size_t)run_op[r]].q[0];
+    o = FOp{};
+    o.type = F_G1;
+    o.t = q;
+    o.term = tm;
+    for (int k = 0; k < 4; ++k) o.m0[k] = W[r][(size_t)k];
+  }
+  fold_diagonals_back(out.ops, n);
+  for (size_t i = 0; i < pars.size(); ++i) {
+    out.recs[i].par = (int32_t)out.pars.size();
+    out.recs[i].npar = (int32_t)pars[i].size();
+    out.pars.insert(out.pars.end(), pars[i].begin(), pars[i].end());
+  }
+  return QS_OK;
+}
+
+// The adjoint sweep over gates [g0, g1) fused into tile passes: the tile planner
+// splits the ops of adjoint_ops (an op keeps its order with the ops that share a
+// qubit), and each pass runs the adjoint pass kernel on psi = st->data and lam, its
+// per-tile sums reduced into dth.
 template <typename R>
 qs_status adjoint_tiled_t(State* st, void* lam, const qs_gate* gates, size_t g0, size_t g1, double* dth) {
   const int n = st->n;
@@ -616,88 +767,64 @@ qs_status adjoint_tiled_t(State* st, void* lam, const qs_gate* gates, size_t g0,
     set_error("fused adjoint needs n >= %d", kTileBits);
     return QS_EUNSUPPORTED;
   }
-  std::vector<qs_gate> bw;
-  std::vector<int> slot;
-  for (size_t g = g1; g-- > g0;) {
-    const qs_gate& G = gates[g];
-    cd U[16], Ud[16];
-    int dim = 0;
-    gate_matrix(G, U, &dim);
-    for (int r = 0; r < dim; ++r)
-      for (int c = 0; c < dim; ++c) Ud[r * dim + c] = std::conj(U[c * dim + r]);
-    auto as_gate = [&](const cd* m) {
-      qs_gate x;
-      std::memset(&x, 0, sizeof(x));
-      x.kind = dim == 2 ? QS_MAT1 : QS_MAT2;
-      x.q[0] = G.q[0];
-      x.q[1] = dim == 2 ? 0 : G.q[1];
-      for (int i = 0; i < dim * dim; ++i) {
-        x.m[2 * i] = m[i].real();
-        x.m[2 * i + 1] = m[i].imag();
-      }
-      return x;
-    };
-    const int np = gate_nparams(G.kind);
-    for (int p = 0; p < np; ++p) {
-      cd dU[16], M[16];
-      gate_dmatrix(G, p, dU);
-      for (int r = 0; r < dim; ++r)
-        for (int c = 0; c < dim; ++c) {
-          cd acc = 0;
-          for (int k = 0; k < dim; ++k) acc += dU[r * dim + k] * Ud[k * dim + c];
-          M[r * dim + c] = acc;
-        }
-      bw.push_back(as_gate(M));
-      slot.push_back((int)(3 * g + p));
-    }
-    bw.push_back(as_gate(Ud));
-    slot.push_back(-1);
-  }
-  std::vector<FOp> fops;
-  std::vector<int> vmap;
-  build_fused_ops(bw.data(), bw.size(), n, fops, vmap, /*fuse=*/false, /*relabel=*/false);
-  if (fops.size() != bw.size()) {
-    set_error("adjoint op list changed size");
-    return QS_EUNSUPPORTED;
-  }
-  for (size_t i = 0; i < fops.size(); ++i) {
-    fops[i].term = slot[i];
-    if (slot[i] >= 0 && fops[i].type != F_G1 && fops[i].type != F_D) {
-      set_error("derivative matrix of gate %d is not a one-qubit or diagonal op", slot[i] / 3);
-      return QS_EUNSUPPORTED;
-    }
-  }
+  AdjointOps ad;
+  qs_status s = adjoint_ops(gates, g0, g1, n, ad);
+  if (s != QS_OK) return s;
+  std::vector<int> vmap(n);
   for (int q = 0; q < n; ++q) vmap[q] = q;
   Plan pl;
-  plan_circuit(fops, n, vmap, pl, TileLimits<R>::kMaxOps, kMaxTileStages);
+  std::vector<TermRec> recs;            // of every pass in turn
+  std::vector<size_t> rec_off;          // per step, one past the last at the end
+  std::vector<int> nsums;               // per step
+  int most = 0;
+  // a pass holds at most kMaxOps sums (its shared memory, and the partials): a plan that exceeds it
+  // is made again with passes that cannot
+  for (int cap : {TileLimits<R>::kMaxOps, TileLimits<R>::kMaxOps / 4}) {
+    plan_circuit(ad.ops, n, vmap, pl, cap, kMaxTileStages);
+    recs.clear();
+    rec_off.clear();
+    nsums.clear();
+    most = 0;
+    for (const PlanStep& step : pl.steps) {
+      rec_off.push_back(recs.size());
+      int ns = 0;
+      if (step.kind == PlanStep::TILE) {
+        const TilePass& pass = pl.passes[step.index];
+        for (int s2 = 0; s2 < pass.n_stages; ++s2) {
+          const TileStage& ts = pl.stages[pass.stage_begin + s2];
+          for (int o = ts.op_begin; o < ts.op_end; ++o) {
+            const int t = pl.tile_fops[o].term;
+            if (t < 0) continue;
+            recs.push_back(ad.recs[(size_t)t]);
+            recs.back().sum = ns;
+            ns += recs.back().nsum;
+          }
+        }
+      }
+      nsums.push_back(ns);
+      most = std::max(most, ns);
+    }
+    rec_off.push_back(recs.size());
+    if (most <= TileLimits<R>::kMaxOps) break;
+  }
   if (!pl.remaps.empty()) {
     set_error("adjoint plan needs a remap");
     return QS_EUNSUPPORTED;
   }
   const uint64_t tiles = 1ull << (n - kTileBits);
-  const size_t pbytes = sizeof(R) * tiles * TileLimits<R>::kMaxOps;
+  const size_t pbytes = sizeof(R) * tiles * (size_t)std::max(most, 1);
   void* partial = dev_alloc(st, pbytes);
   if (!partial) {
     set_error("adjoint partials allocation failed");
     return QS_ENOMEM;
   }
-  // the term slots of every pass, uploaded once
-  std::vector<int> slots_all;
-  std::vector<size_t> slot_off;
-  for (const PlanStep& step : pl.steps) {
-    slot_off.push_back(slots_all.size());
-    if (step.kind != PlanStep::TILE) continue;
-    const TilePass& pass = pl.passes[step.index];
-    for (int s2 = 0; s2 < pass.n_stages; ++s2) {
-      const TileStage& ts = pl.stages[pass.stage_begin + s2];
-      for (int o = ts.op_begin; o < ts.op_end; ++o)
-        if (pl.tile_fops[o].term >= 0) slots_all.push_back(pl.tile_fops[o].term);
-    }
-  }
+  // the records and derivatives of every pass, uploaded once
   std::vector<unsigned char> blob;
-  const size_t off_slots = put(blob, slots_all.data(), slots_all.size());
-  qs_status s = upload(st, blob);
-  const int* slots_dev = (const int*)((unsigned char*)st->opbuf + off_slots);
+  const size_t off_recs = put(blob, recs.data(), recs.size());
+  const size_t off_pars = put(blob, ad.pars.data(), ad.pars.size());
+  s = upload(st, blob);
+  const TermRec* recs_dev = (const TermRec*)((unsigned char*)st->opbuf + off_recs);
+  const TermPar* pars_dev = (const TermPar*)((unsigned char*)st->opbuf + off_pars);
   std::unique_ptr<TileParams<R>> tp(new TileParams<R>());
   for (size_t si = 0; si < pl.steps.size() && s == QS_OK; ++si) {
     const PlanStep& step = pl.steps[si];
@@ -706,12 +833,12 @@ qs_status adjoint_tiled_t(State* st, void* lam, const qs_gate* gates, size_t g0,
       std::memset(tp.get(), 0, sizeof(TileParams<R>));
       tp->pass = pass;
       const int op0 = pl.stages[pass.stage_begin].op_begin;
-      int nterm = 0;
+      size_t rec = rec_off[si];
       for (int s2 = 0; s2 < pass.n_stages; ++s2) {
         TileStage ts = pl.stages[pass.stage_begin + s2];
         for (int o = ts.op_begin; o < ts.op_end; ++o) {
           TileOp<R> t = to_tile<R>(pl, (size_t)o);
-          t.term = pl.tile_fops[o].term >= 0 ? (int16_t)nterm++ : (int16_t)-1;
+          t.term = pl.tile_fops[o].term >= 0 ? (int16_t)recs[rec++].sum : (int16_t)-1;
           tp->ops[o - op0] = t;
         }
         ts.op_begin -= op0;
@@ -719,8 +846,10 @@ qs_status adjoint_tiled_t(State* st, void* lam, const qs_gate* gates, size_t g0,
         tp->stages[s2] = ts;
       }
       tp->pass.stage_begin = 0;
-      s = launch_adjoint_pass(st, lam, tp.get(), partial, nterm);
-      if (s == QS_OK) s = launch_term_reduce(st, partial, nterm, slots_dev + slot_off[si], dth);
+      s = launch_adjoint_pass(st, lam, tp.get(), partial, nsums[si]);
+      if (s == QS_OK)
+        s = launch_term_reduce(st, partial, nsums[si], recs_dev + rec_off[si], (int)(rec_off[si + 1] - rec_off[si]),
+                               pars_dev, dth);
     } else if (step.kind == PlanStep::PLAIN) {
       PlainOp<R> p = to_plain<R>(pl.plain_fops[step.index]);
       s = launch_plain_op(st, &p, p.type);

@@ -20,5 +20,10 @@ void merge_one_qubit_ops(std::vector<FOp>& ops, int n, std::vector<int>* group);
 // The same merge without moving the ops: on return (*into)[i] is the index of the
 // later op that op i was merged into, or -1 for the ops that remain (in order).
 void mark_one_qubit_merges(std::vector<FOp>& ops, int n, std::vector<int>* into);
+// Multiplies diagonal ops without a derivative term into the nearest earlier op that acts
+// non-diagonally on one of their qubits, where that is a one-qubit op whose choice bit (if it has
+// one) is the other qubit: everything in between is diagonal on the diagonal's qubits or misses them.
+// A derivative term of that op is taken before the op is applied, so it is not affected.
+void fold_diagonals_back(std::vector<FOp>& ops, int n);
 
 }  // namespace qs

@@ -9,7 +9,8 @@
 // it runs in fused tile passes (adjoint_pass_kernel: a tile of both states in
 // registers, the U^dagger and derivative terms of all of a pass's gates in one
 // read+write of psi and lambda; dL/dt = 2 Re <lambda_g | G psi_g> with
-// G = (dU/dt) U^dagger).  Otherwise one kernel per gate computes
+// G = (dU/dt) U^dagger, and for a run of one-qubit gates on a qubit all of these
+// from the same four inner products).  Otherwise one kernel per gate computes
 // psi_{g-1} = U_g^dagger psi_g, the derivative terms (fp64 block partials) and
 // lambda_{g-1} = U_g^dagger lambda_g.
 // Rotation derivatives follow from R(t) = exp(-i t sigma/2)

@@ -89,7 +89,8 @@ struct FOp {
   cd m0[4], m1[4]; // G1/G1C matrices U[out][in]
   cd d[4];         // D: entries, index 2*bit_a + bit_b (or bit_a when b < 0)
   cd g[16];        // G2 4x4
-  int term = -1;   // adjoint sweep: derivative-term slot (the op's matrix is dU/dt U^dagger, not applied)
+  int term = -1;   // adjoint sweep: derivative-term record (a diagonal is dU/dt U^dagger and not applied;
+                   // a one-qubit op is applied, after the products of TermRec are summed)
 };
 
 // Converts gates into fused ops.  vmap_out[q] = virtual qubit that holds logical
@@ -304,11 +305,24 @@ qs_status launch_tile_pass(State* st, const void* params);
 // matrix that is not a one-qubit or diagonal op.  Synchronises the stream.
 qs_status adjoint_tiled(State* st, void* lam, const qs_gate* gates, size_t g0, size_t g1, double* dth);
 // adjoint sweep over one tile pass: st->data = psi, lam the adjoint state, params
-// a TileParams image whose ops carry term indices; partial: tiles x nterm values
-// in the state's precision
-qs_status launch_adjoint_pass(State* st, void* lam, const void* params, void* partial, int nterm);
-// dth[slots[i]] += 2 sum over tiles of partial[tile][i]
-qs_status launch_term_reduce(State* st, const void* partial, int nterm, const int* slots, double* dth);
+// a TileParams image whose ops carry the index of their first sum; partial: tiles x
+// nsum values in the state's precision
+qs_status launch_adjoint_pass(State* st, void* lam, const void* params, void* partial, int nsum);
+// What one term op sums over the state, and the derivatives that follow.  A diagonal G: one sum,
+// Re <lambda|G psi>.  A one-qubit op on qubit q: with M_ab = sum conj(lambda_a) psi_b over the
+// other qubits (a, b the values of q), Im M_00, Im M_11, Re(M_01 - M_10) and Im(M_01 + M_10); an
+// anti-Hermitian G on q (dU/dt U^dagger of a unitary U) has Re <lambda|G psi> = c . these with
+// c = (-Im G_00, -Im G_11, Re G_01, -Im G_01).
+struct TermRec {
+  int32_t sum, nsum;   // first sum of the pass's, 1 or 4 of them
+  int32_t par, npar;   // derivatives
+};
+struct TermPar {
+  int64_t slot;        // dth[slot] += 2 sum_k c[k] sum_k
+  double c[4];
+};
+qs_status launch_term_reduce(State* st, const void* partial, int nsum, const TermRec* recs, int nrec,
+                             const TermPar* pars, double* dth);
 qs_status launch_plain_op(State* st, const void* op_dev, int type);
 qs_status launch_small(State* st, const void* ops_dev, int nops);
 qs_status launch_remap(State* st, const RemapDesc& desc);

@@ -286,6 +286,24 @@ void build_fused_ops(const qs_gate* gates, size_t ngates, int n, std::vector<FOp
   }
 }
 
+void fold_diagonals_back(std::vector<FOp>& ops, int n) {
+  std::vector<int> last(n, -1);   // per qubit, the latest op acting non-diagonally on it
+  size_t w = 0;
+  for (size_t i = 0; i < ops.size(); ++i) {
+    const FOp& o = ops[i];
+    if (o.type == F_D && o.term < 0) {
+      const int before = std::max(last[o.a], o.b >= 0 ? last[o.b] : -1);
+      if (before >= 0 && fold_into(o, ops[(size_t)before], /*after=*/true)) continue;
+    }
+    if (w != i) ops[w] = o;
+    const uint64_t m = nd_mask(ops[w]);
+    for (int q = 0; q < n; ++q)
+      if ((m >> q) & 1) last[q] = (int)w;
+    ++w;
+  }
+  ops.resize(w);
+}
+
 void mark_one_qubit_merges(std::vector<FOp>& ops, int n, std::vector<int>* into_out) {
   const size_t m = ops.size();
   std::vector<int>& into = *into_out;   // input op -> the later op it was merged into

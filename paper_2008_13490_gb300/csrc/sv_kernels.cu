@@ -606,65 +606,133 @@ __global__ void __launch_bounds__(kTileThreads)
 // lambda = dL/dpsi^* propagated backwards, dL/dt of a gate's parameter is
 // 2 Re <lambda_g | dU/dt | psi_{g-1}> = 2 Re <lambda_g | G psi_g> with
 // G = (dU/dt) U^dagger, psi_g and lambda_g the states after the gate.  The host
-// lists, for each gate from the last, one op per parameter carrying G (term >= 0)
-// and then U^dagger; the tile planner keeps the order of ops that share a qubit,
-// and a term op commutes with the U^dagger of a gate on other qubits (that unitary
-// cancels from the inner product).  Here a tile of psi and one of lambda stay in
-// registers through the pass: U^dagger ops act on both, a term op adds
-// Re sum_J conj(lambda_J) (G psi)_J over the tile into s_term[term] (warp sums,
-// shared-memory atomics), written per tile to partial[tile][term].
+// lists, from the last gate, runs of one-qubit gates on a qubit as one op: the inner
+// products of TermRec, from which the derivatives of all the run's parameters
+// follow, then the product of the run's U^dagger, applied to both states.  A diagonal
+// gate has one op per parameter carrying G (TK_DIAG with term >= 0, not applied) and
+// then U^dagger.  The tile planner keeps the order of ops that share a qubit, and a
+// term op commutes with the U^dagger of a gate on other qubits (that unitary cancels
+// from the inner product).  Here a tile of psi and one of lambda stay in registers
+// through the pass; an op's sums over the tile go to s_term (warp sums, shared-memory
+// atomics), written per tile to partial[tile][sum].
+//
+// The FP32 pipe bounds it (24 qubits, 20 layers of three rotations and CZs: 480 runs).  With a term op and a U^dagger per gate, three of each per run, and the CZs as
+// diagonals of their own the sweep took 40.1 ms, now 9.9 (11 passes, now 8).
 
-// Re sum over this thread's 16 amplitudes of conj(l) (G p), G the op's matrix
+// The sums over this thread's amplitudes that an op of a TermRec takes.
 template <typename R>
-__device__ __forceinline__ R term_of_op(const C2<R>* vp, const C2<R>* vl, const TileOp<R>* __restrict__ opp,
-                                        uint64_t tile, int lane, int warp) {
+struct CrossSum {
+  R a0 = 0, a1 = 0, re = 0, im = 0;
+  __device__ __forceinline__ void pair(C2<R> l0, C2<R> l1, C2<R> p0, C2<R> p1) {
+    a0 = fma(l0.x, p0.y, a0);
+    a0 = fma(-l0.y, p0.x, a0);
+    a1 = fma(l1.x, p1.y, a1);
+    a1 = fma(-l1.y, p1.x, a1);
+    re = fma(l0.x, p1.x, re);
+    re = fma(l0.y, p1.y, re);
+    re = fma(-l1.x, p0.x, re);
+    re = fma(-l1.y, p0.y, re);
+    im = fma(l0.x, p1.y, im);
+    im = fma(-l0.y, p1.x, im);
+    im = fma(l1.x, p0.y, im);
+    im = fma(-l1.y, p0.x, im);
+  }
+  // one amplitude of a qubit on a lane bit: own l and p, the partner lane's p (to be finished by lane_end)
+  __device__ __forceinline__ void single(C2<R> l, C2<R> p, C2<R> q) {
+    a0 = fma(l.x, p.y, a0);
+    a0 = fma(-l.y, p.x, a0);
+    re = fma(l.x, q.x, re);
+    re = fma(l.y, q.y, re);
+    im = fma(l.x, q.y, im);
+    im = fma(-l.y, q.x, im);
+  }
+  __device__ __forceinline__ void lane_end(bool b) {
+    a1 = b ? a0 : R(0);
+    a0 = b ? R(0) : a0;
+    re = b ? -re : re;
+  }
+  // adds the warp's sums to dst[0..3]: the four values are spread over lane pairs and quads, then
+  // one value per lane (lane & 3) is summed over the lanes
+  __device__ __forceinline__ void add_to(R* dst, int lane) const {
+    const bool o = lane & 1, t = lane & 2;
+    const R x = (o ? a1 : a0) + __shfl_xor_sync(0xffffffffu, o ? a0 : a1, 1);
+    const R y = (o ? im : re) + __shfl_xor_sync(0xffffffffu, o ? re : im, 1);
+    R z = (t ? y : x) + __shfl_xor_sync(0xffffffffu, t ? x : y, 2);
+#pragma unroll
+    for (int m = 4; m < 32; m <<= 1) z += __shfl_xor_sync(0xffffffffu, z, m);
+    if (lane < 4) atomicAdd(dst + lane, z);
+  }
+};
+
+template <int J, typename R>
+__device__ __forceinline__ void reg_cross(const C2<R>* vp, const C2<R>* vl, CrossSum<R>& s) {
+#pragma unroll
+  for (int r = 0; r < 16; ++r)
+    if (!(r & (1 << J))) s.pair(vl[r], vl[r | (1 << J)], vp[r], vp[r | (1 << J)]);
+}
+
+// lane qubit: the sums and the op (own and partner coefficients o0, p0, or o1, p1 where
+// register bit K is 1; K < 0: one pair) on both states, psi's partner amplitudes fetched once
+template <int K, typename R>
+__device__ __forceinline__ void lane_cross(C2<R>* vp, C2<R>* vl, int mask, C2<R> o0, C2<R> p0, C2<R> o1, C2<R> p1,
+                                           CrossSum<R>& s) {
+#pragma unroll
+  for (int r = 0; r < 16; ++r) {
+    const C2<R> q = shfl_xor_c(vp[r], mask), k = shfl_xor_c(vl[r], mask);
+    s.single(vl[r], vp[r], q);
+    const bool one = K >= 0 && ((r >> (K < 0 ? 0 : K)) & 1);
+    const C2<R> o = one ? o1 : o0, p = one ? p1 : p0;
+    vp[r] = cfma2(o, vp[r], p, q);
+    vl[r] = cfma2(o, vl[r], p, k);
+  }
+}
+
+// a run's op (TK_REG or TK_LANE, term >= 0): its sums to dst, then the op on both states
+template <typename R>
+__device__ __forceinline__ void apply_run(C2<R>* vp, C2<R>* vl, const TileOp<R>* __restrict__ opp, uint64_t tile,
+                                          int lane, int warp, R* dst) {
+  CrossSum<R> s;
+  if (opp->kind == TK_REG) {
+    switch (opp->slot) {
+      case 0: reg_cross<0>(vp, vl, s); break;
+      case 1: reg_cross<1>(vp, vl, s); break;
+      case 2: reg_cross<2>(vp, vl, s); break;
+      default: reg_cross<3>(vp, vl, s); break;
+    }
+    s.add_to(dst, lane);
+    apply_tile_op<R, false>(vp, opp, tile, lane, warp);
+    apply_tile_op<R, false>(vl, opp, tile, lane, warp);
+    return;
+  }
+  const int mask = 1 << opp->slot;
+  const bool b = (lane & mask) != 0;
+  const uint8_t csrc = opp->csrc, cbit = opp->cbit;
+  const C2<R> o0 = csel(b, opp->m0[3], opp->m0[0]), p0 = csel(b, opp->m0[2], opp->m0[1]);
+  const C2<R> o1 = csel(b, opp->m1[3], opp->m1[0]), p1 = csel(b, opp->m1[2], opp->m1[1]);
+  if (csrc == CS_REG) {
+    switch (cbit) {
+      case 0: lane_cross<0>(vp, vl, mask, o0, p0, o1, p1, s); break;
+      case 1: lane_cross<1>(vp, vl, mask, o0, p0, o1, p1, s); break;
+      case 2: lane_cross<2>(vp, vl, mask, o0, p0, o1, p1, s); break;
+      default: lane_cross<3>(vp, vl, mask, o0, p0, o1, p1, s); break;
+    }
+  } else {
+    const bool c = csrc != CS_NONE && src_bit<R>(csrc, cbit, tile, lane, warp);
+    lane_cross<-1>(vp, vl, mask, csel(c, o1, o0), csel(c, p1, p0), o1, p1, s);
+  }
+  s.lane_end(b);
+  s.add_to(dst, lane);
+}
+
+// Re sum over this thread's 16 amplitudes of conj(l) (G p), G the diagonal d[2 bit_a + bit_b]
+template <typename R>
+__device__ __forceinline__ R term_of_diag(const C2<R>* vp, const C2<R>* vl, const TileOp<R>* __restrict__ opp,
+                                          uint64_t tile, int lane, int warp) {
   C2<R> g[4];
 #pragma unroll
   for (int i = 0; i < 4; ++i) g[i] = opp->m0[i];
   R t = 0;
   auto dotre = [](C2<R> a, C2<R> b) { return fma(a.x, b.x, a.y * b.y); };   // Re conj(a) b
-  if (opp->kind == TK_REG) {
-    // pairs (r, r | 2^k) of register slot k; a switch keeps register indices constant
-    switch (opp->slot) {
-      case 0:
-#pragma unroll
-        for (int r = 0; r < 16; ++r) {
-          if (r & 1) continue;
-          t += dotre(vl[r], cfma2(g[0], vp[r], g[1], vp[r | 1])) + dotre(vl[r | 1], cfma2(g[2], vp[r], g[3], vp[r | 1]));
-        }
-        break;
-      case 1:
-#pragma unroll
-        for (int r = 0; r < 16; ++r) {
-          if (r & 2) continue;
-          t += dotre(vl[r], cfma2(g[0], vp[r], g[1], vp[r | 2])) + dotre(vl[r | 2], cfma2(g[2], vp[r], g[3], vp[r | 2]));
-        }
-        break;
-      case 2:
-#pragma unroll
-        for (int r = 0; r < 16; ++r) {
-          if (r & 4) continue;
-          t += dotre(vl[r], cfma2(g[0], vp[r], g[1], vp[r | 4])) + dotre(vl[r | 4], cfma2(g[2], vp[r], g[3], vp[r | 4]));
-        }
-        break;
-      default:
-#pragma unroll
-        for (int r = 0; r < 16; ++r) {
-          if (r & 8) continue;
-          t += dotre(vl[r], cfma2(g[0], vp[r], g[1], vp[r | 8])) + dotre(vl[r | 8], cfma2(g[2], vp[r], g[3], vp[r | 8]));
-        }
-    }
-    return t;
-  }
-  if (opp->kind == TK_LANE) {
-    const int mask = 1 << opp->slot;
-    const bool b = (lane & mask) != 0;
-    const C2<R> o = csel(b, g[3], g[0]), q = csel(b, g[2], g[1]);   // own and partner coefficients
-#pragma unroll
-    for (int r = 0; r < 16; ++r) t += dotre(vl[r], cfma2(o, vp[r], q, shfl_xor_c(vp[r], mask)));
-    return t;
-  }
-  // TK_DIAG: (G p)_J = d[2 bit_a + bit_b] p_J
   const uint8_t csrc = opp->csrc, cbit = opp->cbit, dsrc = opp->dsrc, dbit = opp->dbit;
   const bool two = dsrc != CS_NONE;
   const int ua = csrc == CS_REG ? 0 : src_bit<R>(csrc, cbit, tile, lane, warp);
@@ -683,7 +751,7 @@ __device__ __forceinline__ R term_of_op(const C2<R>* vp, const C2<R>* vl, const 
 template <typename R, bool G2>
 __global__ void __launch_bounds__(kTileThreads, sizeof(R) == 4 ? 2 : 1)
     adjoint_pass_kernel(C2<R>* __restrict__ psi, C2<R>* __restrict__ lam,
-                        const __grid_constant__ TileParams<R> P, R* __restrict__ partial, int nterm) {
+                        const __grid_constant__ TileParams<R> P, R* __restrict__ partial, int nsum) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C2<R>* smp = reinterpret_cast<C2<R>*>(smem_raw);
   C2<R>* sml = smp + (1 << kTileBits);
@@ -700,7 +768,7 @@ __global__ void __launch_bounds__(kTileThreads, sizeof(R) == 4 ? 2 : 1)
     s_base = base;
   }
   if (tid < kTileBits) s_pos[tid] = P.pass.pos[tid];
-  for (int i = tid; i < nterm; i += kTileThreads) s_term[i] = R(0);
+  for (int i = tid; i < nsum; i += kTileThreads) s_term[i] = R(0);
   __syncthreads();
   const uint64_t base = s_base;
   uint64_t loff = 0;
@@ -772,8 +840,13 @@ __global__ void __launch_bounds__(kTileThreads, sizeof(R) == 4 ? 2 : 1)
     }
     for (int o = cur.op_begin; o < cur.op_end;) {
       const TileOp<R>* op = ops + o;
+      if (op->term >= 0 && op->kind != TK_DIAG) {
+        apply_run<R>(vp, vl, op, tile, lane, warp, s_term + op->term);
+        ++o;
+        continue;
+      }
       if (op->term >= 0) {
-        R t = term_of_op<R>(vp, vl, op, tile, lane, warp);
+        R t = term_of_diag<R>(vp, vl, op, tile, lane, warp);
 #pragma unroll
         for (int m = 16; m > 0; m >>= 1) t += __shfl_xor_sync(0xffffffffu, t, m);
         if (lane == 0) atomicAdd(&s_term[op->term], t);
@@ -816,19 +889,30 @@ __global__ void __launch_bounds__(kTileThreads, sizeof(R) == 4 ? 2 : 1)
     }
   }
   __syncthreads();
-  for (int i = tid; i < nterm; i += kTileThreads) partial[(size_t)tile * nterm + i] = s_term[i];
+  for (int i = tid; i < nsum; i += kTileThreads) partial[(size_t)tile * nsum + i] = s_term[i];
 }
 
-// dth[slots[i]] += 2 sum over tiles of partial[tile][i] (FP64, one block per term)
+// the sums of a record over the tiles (FP64, one block per record) and the derivatives they give
 template <typename R>
 __global__ void __launch_bounds__(256)
-    term_reduce_kernel(const R* __restrict__ partial, uint64_t tiles, int nterm,
-                       const int* __restrict__ slots, double* __restrict__ dth) {
-  const int i = blockIdx.x;
-  double acc = 0.0;
-  for (uint64_t t = threadIdx.x; t < tiles; t += blockDim.x) acc += (double)partial[t * nterm + i];
-  const double tot = block_sum(acc);
-  if (threadIdx.x == 0) dth[slots[i]] += 2.0 * tot;
+    term_reduce_kernel(const R* __restrict__ partial, uint64_t tiles, int nsum, const TermRec* __restrict__ recs,
+                       const TermPar* __restrict__ pars, double* __restrict__ dth) {
+  const TermRec r = recs[blockIdx.x];
+  double acc[4] = {0.0, 0.0, 0.0, 0.0};
+  for (uint64_t t = threadIdx.x; t < tiles; t += blockDim.x) {
+    const R* p = partial + t * nsum + r.sum;
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      if (k < r.nsum) acc[k] += (double)p[k];
+  }
+#pragma unroll
+  for (int k = 0; k < 4; ++k)
+    if (k < r.nsum) acc[k] = block_sum(acc[k]);
+  if (threadIdx.x) return;
+  for (int i = r.par; i < r.par + r.npar; ++i) {
+    const TermPar& q = pars[i];
+    dth[q.slot] += 2.0 * (q.c[0] * acc[0] + q.c[1] * acc[1] + q.c[2] * acc[2] + q.c[3] * acc[3]);
+  }
 }
 
 // ------------------------------------------------------------------ plain per-gate
@@ -1404,35 +1488,36 @@ qs_status launch_tile_pass(State* st, const void* params) {
 }
 
 template <typename R, bool G2>
-static qs_status adjoint_launch_t(State* st, void* lam, const TileParams<R>& P, void* partial, int nterm) {
+static qs_status adjoint_launch_t(State* st, void* lam, const TileParams<R>& P, void* partial, int nsum) {
   const uint64_t tiles = 1ull << (st->n - kTileBits);
   const size_t smem = 2 * (sizeof(C2<R>) << kTileBits);
   qs_status s = set_smem(adjoint_pass_kernel<R, G2>, smem);
   if (s != QS_OK) return s;
   adjoint_pass_kernel<R, G2><<<(unsigned)tiles, kTileThreads, smem, st->stream>>>(
-      (C2<R>*)st->data, (C2<R>*)lam, P, (R*)partial, nterm);
+      (C2<R>*)st->data, (C2<R>*)lam, P, (R*)partial, nsum);
   QS_CUDA(cudaGetLastError());
   return QS_OK;
 }
 
-qs_status launch_adjoint_pass(State* st, void* lam, const void* params, void* partial, int nterm) {
+qs_status launch_adjoint_pass(State* st, void* lam, const void* params, void* partial, int nsum) {
   if (st->prec == QS_C64) {
     const TileParams<float>& P = *(const TileParams<float>*)params;
-    return pass_has_g2(P) ? adjoint_launch_t<float, true>(st, lam, P, partial, nterm)
-                          : adjoint_launch_t<float, false>(st, lam, P, partial, nterm);
+    return pass_has_g2(P) ? adjoint_launch_t<float, true>(st, lam, P, partial, nsum)
+                          : adjoint_launch_t<float, false>(st, lam, P, partial, nsum);
   }
   const TileParams<double>& P = *(const TileParams<double>*)params;
-  return pass_has_g2(P) ? adjoint_launch_t<double, true>(st, lam, P, partial, nterm)
-                        : adjoint_launch_t<double, false>(st, lam, P, partial, nterm);
+  return pass_has_g2(P) ? adjoint_launch_t<double, true>(st, lam, P, partial, nsum)
+                        : adjoint_launch_t<double, false>(st, lam, P, partial, nsum);
 }
 
-qs_status launch_term_reduce(State* st, const void* partial, int nterm, const int* slots, double* dth) {
-  if (nterm <= 0) return QS_OK;
+qs_status launch_term_reduce(State* st, const void* partial, int nsum, const TermRec* recs, int nrec,
+                             const TermPar* pars, double* dth) {
+  if (nrec <= 0) return QS_OK;
   const uint64_t tiles = 1ull << (st->n - kTileBits);
   if (st->prec == QS_C64)
-    term_reduce_kernel<float><<<nterm, 256, 0, st->stream>>>((const float*)partial, tiles, nterm, slots, dth);
+    term_reduce_kernel<float><<<nrec, 256, 0, st->stream>>>((const float*)partial, tiles, nsum, recs, pars, dth);
   else
-    term_reduce_kernel<double><<<nterm, 256, 0, st->stream>>>((const double*)partial, tiles, nterm, slots, dth);
+    term_reduce_kernel<double><<<nrec, 256, 0, st->stream>>>((const double*)partial, tiles, nsum, recs, pars, dth);
   QS_CUDA(cudaGetLastError());
   return QS_OK;
 }
