@@ -122,7 +122,8 @@ struct alignas(16) TileOp {
   uint8_t dsrc;    // TK_DIAG: source of bit b (CS_NONE for one-qubit diagonals)
   uint8_t dbit;
   int16_t term;    // adjoint pass: index of the derivative term this op forms, or -1
-  uint8_t pad[8];
+  uint8_t pad[8];  // TK_CP: [0], [1] (tile_cp.h); TK_REG/TK_LANE: [2] = 1 if every matrix
+                   // entry is real, 2 if the matrix is [1 1; 1 -1] (no choice bit)
   C2<R> m0[4];     // matrix (choice bit 0) or diagonal d[0..3]
   C2<R> m1[4];     // matrix (choice bit 1)
 };
@@ -163,7 +164,9 @@ struct TileParams {
   TileOp<R> ops[TileLimits<R>::kMaxOps];
   const C2<R>* tabs;            // the pass's run tables (device; forward passes with TK_RUN)
   int32_t n_jobs;               // run prologue jobs (RunJob, tile_cp.h)
+  int32_t n_tjobs;              // thread jobs
   uint8_t jobs[64 * 8];
+  uint8_t tjobs[64 * 8];
 };
 
 // Device-side plain op (one launch per op; also the small-state kernel's op).

@@ -83,6 +83,15 @@ void d_restrict(const FOp& D, int t, int v, cd* d0, cd* d1) {
   }
 }
 
+bool is_real(const FOp& o) {
+  bool real = true;
+  for (int k = 0; k < 4; ++k) {
+    if (o.type == F_D) real = real && (o.d[k].imag() == 0.0);
+    else real = real && o.m0[k].imag() == 0.0 && (o.type != F_G1C || o.m1[k].imag() == 0.0);
+  }
+  return real;
+}
+
 // Try to fold diagonal op D into G (a G1 or G1C acting non-diagonally on a
 // qubit of D).  after = true: D acts after G (D G); else D acts before G (G D).
 bool fold_into(const FOp& D, FOp& G, bool after) {
@@ -90,6 +99,10 @@ bool fold_into(const FOp& D, FOp& G, bool after) {
   bool t_in = (t == D.a) || (t == D.b);
   if (!t_in) return false;
   int other = (D.b < 0) ? -1 : (t == D.a ? D.b : D.a);
+  // A real op (H, RY, X, CNOT) stays real: it takes half the instructions, and the phase joins a
+  // run of its own kind at less than it would add here (30-qubit Fourier transform: 52.3 ms with
+  // the phase folded in, 46.1 without).
+  if (other >= 0 && (G.type == F_G1 || G.type == F_G1C) && is_real(G) && !is_real(D)) return false;
   if (G.type == F_G1) {
     if (other < 0) {
       cd d0, d1;
@@ -542,11 +555,21 @@ void plan_circuit(const std::vector<FOp>& ops, int n, const std::vector<int>& vm
       int nR = 0;
       uint64_t snd = 0, sd = 0;
       std::vector<int> stage_ops, later;
+      // Diagonals wait until an op acts non-diagonally on one of their qubits, or to the pass's
+      // end: what stands between two such ops is then one run, and the phases between a qubit
+      // of the tile and the qubits outside it are multiplied once per pass.  (With the run code of
+      // sv_kernels.cu, a 30-qubit Fourier transform: 55.4 ms when each phase stood at its place,
+      // 52.3 so.)
+      std::vector<int> held;
       for (int idx : pending) {
         const FOp& o = pv[idx];
         uint64_t ndq = nd_mask(o), dq = d_mask(o);
         bool conflict = (ndq & (snd | sd)) || (dq & snd);
         bool ok = false;
+        if (!conflict && o.type == F_D && o.term < 0) {
+          held.push_back(idx);
+          continue;
+        }
         if (!conflict && o.type == F_G2) {
           // both qubits on lanes or in this stage's registers
           const int la = enc.local_of_phys[l2p[o.a]], lb = enc.local_of_phys[l2p[o.b]];
@@ -579,12 +602,27 @@ void plan_circuit(const std::vector<FOp>& ops, int n, const std::vector<int>& vm
             }
           }
         }
-        if (ok) stage_ops.push_back(idx);
-        else {
+        if (ok) {
+          size_t w = 0;
+          for (int h : held) {
+            if (d_mask(pv[(size_t)h]) & ndq) stage_ops.push_back(h);
+            else held[w++] = h;
+          }
+          held.resize(w);
+          stage_ops.push_back(idx);
+        } else {
           snd |= ndq;
           sd |= dq;
           later.push_back(idx);
         }
+      }
+      later.insert(later.end(), held.begin(), held.end());
+      std::sort(later.begin(), later.end());
+      bool nd_left = false;
+      for (int idx : later) nd_left = nd_left || pv[(size_t)idx].type != F_D;
+      if (!nd_left) {
+        stage_ops.insert(stage_ops.end(), later.begin(), later.end());
+        later.clear();
       }
       // complete the register set (prefer targets needed next)
       for (int idx : later) {

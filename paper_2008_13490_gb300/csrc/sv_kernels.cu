@@ -17,6 +17,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cstddef>
 #include <cstring>
 
 #include "dev_common.cuh"
@@ -58,6 +59,45 @@ __device__ __forceinline__ void lane_gate_choice(C2<R>* v, int mask, C2<R> o0, C
     const C2<R> q = shfl_xor_c(v[r], mask);
     if ((r >> K) & 1) v[r] = cfma2(o1, v[r], p1, q);
     else v[r] = cfma2(o0, v[r], p0, q);
+  }
+}
+
+// ---- ops whose matrices are real (H, RY, X, CNOT): a product with each part, two packed FP32
+// instructions per output amplitude in place of four; the values are those of cfma2
+
+template <typename R>
+__device__ __forceinline__ C2<R> rfma2(R m0, C2<R> a, R m1, C2<R> b) {
+  return C2<R>{fma(m1, b.x, m0 * a.x), fma(m1, b.y, m0 * a.y)};
+}
+template <>
+__device__ __forceinline__ C2<float> rfma2<float>(float m0, C2<float> a, float m1, C2<float> b) {
+  const float2 r = __ffma2_rn(make_float2(m1, m1), make_float2(b.x, b.y),
+                              __fmul2_rn(make_float2(m0, m0), make_float2(a.x, a.y)));
+  return C2<float>{r.x, r.y};
+}
+
+// K < 0: the matrix m0; else m1 where register bit K is 1
+template <int J, int K, typename R>
+__device__ __forceinline__ void reg_gate_real(C2<R>* v, const R* m0, const R* m1) {
+#pragma unroll
+  for (int r = 0; r < 16; ++r) {
+    if (r & (1 << J)) continue;
+    const R* m = K >= 0 && ((r >> (K < 0 ? 0 : K)) & 1) ? m1 : m0;
+    const C2<R> a = v[r], b = v[r | (1 << J)];
+    v[r] = rfma2(m[0], a, m[1], b);
+    v[r | (1 << J)] = rfma2(m[2], a, m[3], b);
+  }
+}
+
+// [1 1; 1 -1] (a Hadamard gate but for its factor, which the host gives to one op of several)
+template <int J, typename R>
+__device__ __forceinline__ void reg_butterfly(C2<R>* v) {
+#pragma unroll
+  for (int r = 0; r < 16; ++r) {
+    if (r & (1 << J)) continue;
+    const C2<R> a = v[r], b = v[r | (1 << J)];
+    v[r] = C2<R>{a.x + b.x, a.y + b.y};
+    v[r | (1 << J)] = C2<R>{a.x - b.x, a.y - b.y};
   }
 }
 
@@ -184,15 +224,87 @@ __device__ __forceinline__ int src_bit(uint8_t src, uint8_t bit, uint64_t tile, 
 
 // G2: the pass holds dense two-qubit ops (a kernel variant of its own, so that
 // passes without them keep the leaner code)
-template <typename R, bool G2>
+// REAL: real matrices take their own path
+template <typename R, bool G2, bool REAL = true>
 __device__ __forceinline__ void apply_tile_op(C2<R>* v, const TileOp<R>* __restrict__ opp,
                                               uint64_t tile, int lane, int warp) {
-  const uint8_t kind = opp->kind, slot = opp->slot, csrc = opp->csrc, cbit = opp->cbit;
+  // (the first 16 bytes with one load: kind, slot, csrc, cbit | dsrc, dbit, term | pad[0..3] | pad[4..7])
+  const uint4 hdr = *reinterpret_cast<const uint4*>(opp);
+  const uint32_t kind = hdr.x & 0xffu, slot = (hdr.x >> 8) & 0xffu, csrc = (hdr.x >> 16) & 0xffu, cbit = hdr.x >> 24;
   if constexpr (G2) {
     if (kind == TK_G2) {   // reads its continuation opp[1]
       apply_g2(v, opp, lane);
       return;
     }
+  }
+  if (REAL && (hdr.z & 0xff0000u)) {   // pad[2]: a real TK_REG or TK_LANE op
+    R a[4], b[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      a[i] = opp->m0[i].x;
+      b[i] = opp->m1[i].x;
+    }
+    const bool in_reg = csrc == CS_REG;
+    // [1 1; 1 -1] (beside the dense two-qubit code it costs registers, and with them a CTA per SM)
+    if (!G2 && (hdr.z & 0xff0000u) == 0x20000u) {
+      if (kind == TK_REG) {
+        switch (slot) {
+          case 0: reg_butterfly<0>(v); break;
+          case 1: reg_butterfly<1>(v); break;
+          case 2: reg_butterfly<2>(v); break;
+          default: reg_butterfly<3>(v); break;
+        }
+        return;
+      }
+      const int mask = 1 << slot;
+      const R sign = (lane & mask) ? R(-1) : R(1);
+#pragma unroll
+      for (int r = 0; r < 16; ++r) {
+        const C2<R> q = shfl_xor_c(v[r], mask);
+        v[r] = C2<R>{fma(sign, v[r].x, q.x), fma(sign, v[r].y, q.y)};
+      }
+      return;
+    }
+    if (!in_reg && csrc != CS_NONE && src_bit<R>(csrc, cbit, tile, lane, warp)) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) a[i] = b[i];
+    }
+    if (kind == TK_REG) {
+      switch (in_reg ? slot * 4 + cbit : 16 + slot) {
+        case 1: reg_gate_real<0, 1>(v, a, b); break;
+        case 2: reg_gate_real<0, 2>(v, a, b); break;
+        case 3: reg_gate_real<0, 3>(v, a, b); break;
+        case 4: reg_gate_real<1, 0>(v, a, b); break;
+        case 6: reg_gate_real<1, 2>(v, a, b); break;
+        case 7: reg_gate_real<1, 3>(v, a, b); break;
+        case 8: reg_gate_real<2, 0>(v, a, b); break;
+        case 9: reg_gate_real<2, 1>(v, a, b); break;
+        case 11: reg_gate_real<2, 3>(v, a, b); break;
+        case 12: reg_gate_real<3, 0>(v, a, b); break;
+        case 13: reg_gate_real<3, 1>(v, a, b); break;
+        case 14: reg_gate_real<3, 2>(v, a, b); break;
+        case 16: reg_gate_real<0, -1>(v, a, a); break;
+        case 17: reg_gate_real<1, -1>(v, a, a); break;
+        case 18: reg_gate_real<2, -1>(v, a, a); break;
+        default: reg_gate_real<3, -1>(v, a, a); break;
+      }
+      return;
+    }
+    const int mask = 1 << slot;
+    const bool up = (lane >> slot) & 1;
+    const R o0 = up ? a[3] : a[0], p0 = up ? a[2] : a[1], o1 = up ? b[3] : b[0], p1 = up ? b[2] : b[1];
+    if (!G2 && !in_reg) {   // (registers, as above)
+#pragma unroll
+      for (int r = 0; r < 16; ++r) v[r] = rfma2(o0, v[r], p0, shfl_xor_c(v[r], mask));
+      return;
+    }
+#pragma unroll
+    for (int r = 0; r < 16; ++r) {
+      const C2<R> q = shfl_xor_c(v[r], mask);
+      const bool one = in_reg && ((r >> cbit) & 1);
+      v[r] = rfma2(one ? o1 : o0, v[r], one ? p1 : p0, q);
+    }
+    return;
   }
   C2<R> m0[4], m1[4];
 #pragma unroll
@@ -286,13 +398,16 @@ __device__ __forceinline__ void apply_tile_op(C2<R>* v, const TileOp<R>* __restr
 template <typename R>
 struct DiagRun {
   C2<R> s, f0[2], f1[2], f2[2], f3[2];   // compile-time indices only (registers)
+  bool slots;                            // a factor of a register slot was set (the same for the warp)
 
   __device__ __forceinline__ void reset() {
     const C2<R> one{R(1), R(0)};
+    slots = false;
     s = one;
     f0[0] = f0[1] = f1[0] = f1[1] = f2[0] = f2[1] = f3[0] = f3[1] = one;
   }
   __device__ __forceinline__ void fold(int k, C2<R> e0, C2<R> e1) {
+    slots = true;
     switch (k) {
       case 0: f0[0] = cmul(f0[0], e0); f0[1] = cmul(f0[1], e1); break;
       case 1: f1[0] = cmul(f1[0], e0); f1[1] = cmul(f1[1], e1); break;
@@ -353,6 +468,7 @@ struct DiagRun {
     const int ub = rb ? 1 : (int)((ctx >> pb) & 1ull);
     const C2<R> e = csel((ua & ub) != 0, p, one);
     if (ra || rb) {
+      slots = true;
       switch (ra ? cbit : dbit) {
         case 0: f0[1] = cmul(f0[1], e); break;
         case 1: f1[1] = cmul(f1[1], e); break;
@@ -363,74 +479,17 @@ struct DiagRun {
       s = cmul(s, e);
     }
   }
-  // TK_RUN (tile_cp.h): the residual entries, the CTA's prologue factors U of the
-  // run's jobs, and the (lane, warp) / register tables of the pass (lw = warp * 32 +
-  // lane)
-  __device__ __forceinline__ void add_run(C2<R>* v, const TileOp<R>* __restrict__ opp, uint64_t ctx, int lw,
-                                          const C2<R>* U, const C2<R>* __restrict__ tabs) {
-    RunHeader h;
-    memcpy(&h, &opp->m0[0], sizeof(h));
-    const RunEntry<R>* __restrict__ e = reinterpret_cast<const RunEntry<R>*>(opp + 1);
-    const C2<R> one{R(1), R(0)};
-    int i = 0;
-    for (const int n = h.n_s; i < n; ++i) {
-      const RunEntry<R> x = e[i];
-      s = cmul(s, csel(((ctx >> x.pa) & (ctx >> x.pb) & 1ull) != 0, x.p, one));
-    }
-    for (const int n = i + h.n_f[0]; i < n; ++i) {
-      const RunEntry<R> x = e[i];
-      f0[1] = cmul(f0[1], csel(((ctx >> x.pa) & 1ull) != 0, x.p, one));
-    }
-    for (const int n = i + h.n_f[1]; i < n; ++i) {
-      const RunEntry<R> x = e[i];
-      f1[1] = cmul(f1[1], csel(((ctx >> x.pa) & 1ull) != 0, x.p, one));
-    }
-    for (const int n = i + h.n_f[2]; i < n; ++i) {
-      const RunEntry<R> x = e[i];
-      f2[1] = cmul(f2[1], csel(((ctx >> x.pa) & 1ull) != 0, x.p, one));
-    }
-    for (const int n = i + h.n_f[3]; i < n; ++i) {
-      const RunEntry<R> x = e[i];
-      f3[1] = cmul(f3[1], csel(((ctx >> x.pa) & 1ull) != 0, x.p, one));
-    }
-    if (h.umask) {
-      int u = h.ubase;
-      if (h.umask & 1) s = cmul(s, U[u++]);
-      if (h.umask & 2) f0[1] = cmul(f0[1], U[u++]);
-      if (h.umask & 4) f1[1] = cmul(f1[1], U[u++]);
-      if (h.umask & 8) f2[1] = cmul(f2[1], U[u++]);
-      if (h.umask & 16) f3[1] = cmul(f3[1], U[u++]);
-    }
-    if (h.tmask) {
-      const C2<R>* __restrict__ T = tabs + h.toff;
-      if (h.tmask & 1) {
-        s = cmul(s, T[lw]);
-        T += kRunTable;
-      }
-      if (h.tmask & 2) {
-        f0[1] = cmul(f0[1], T[lw]);
-        T += kRunTable;
-      }
-      if (h.tmask & 4) {
-        f1[1] = cmul(f1[1], T[lw]);
-        T += kRunTable;
-      }
-      if (h.tmask & 8) {
-        f2[1] = cmul(f2[1], T[lw]);
-        T += kRunTable;
-      }
-      if (h.tmask & 16) {
-        f3[1] = cmul(f3[1], T[lw]);
-        T += kRunTable;
-      }
-      if (h.tmask & 32) {
-#pragma unroll
-        for (int r = 0; r < 16; ++r) v[r] = cmul(v[r], T[r]);
-      }
-    }
-  }
   template <bool TWO = false>
   __device__ __forceinline__ void flush(C2<R>* v, C2<R>* v2 = nullptr) {
+    if (!slots) {
+#pragma unroll
+      for (int r = 0; r < 16; ++r) {
+        v[r] = cmul(v[r], s);
+        if (TWO) v2[r] = cmul(v2[r], s);
+      }
+      reset();
+      return;
+    }
     // D(r) = s f0[r0] f1[r1] f2[r2] f3[r3] as (s f0 f1)[r & 3] * (f2 f3)[r >> 2]
     const C2<R> a0 = cmul(s, f0[0]), a1 = cmul(s, f0[1]);
     const C2<R> lo[4] = {cmul(a0, f1[0]), cmul(a1, f1[0]), cmul(a0, f1[1]), cmul(a1, f1[1])};
@@ -446,11 +505,125 @@ struct DiagRun {
   }
 };
 
+// TK_RUN (tile_cp.h): a diagonal s prod_k f_k^(bit k of r) T[r] over the 16 register indices.
+// U, W: the CTA's factors of the jobs and thread jobs; tabs: the (lane, warp) and register
+// tables of the pass (lw = warp * 32 + lane).  Instruction issue bounds the pass, not HBM (30-qubit
+// Fourier transform: 10.6 ms a pass for 2.5 ms of traffic): a run whose ops share a register slot,
+// as those before a Hadamard on it do, touches the eight amplitudes where it is 1 and no others, and
+// the rest of the diagonal is formed once from lo and hi parts (14.5 ms a pass with the general
+// diagonal of DiagRun for each run, and the tile x thread phases one by one in each thread).
+template <typename R>
+__device__ __forceinline__ C2<R> run_entries(C2<R> f, const RunEntry<R>* __restrict__ e, int n, uint64_t ctx) {
+  const C2<R> one{R(1), R(0)};
+  for (int i = 0; i < n; ++i) {
+    const RunEntry<R> x = e[i];
+    f = cmul(f, csel(((ctx >> x.pa) & 1ull) != 0, x.p, one));
+  }
+  return f;
+}
+// every op has a bit in slot K: the amplitudes where it is 1
+template <int K, typename R>
+__device__ __forceinline__ void run_in_slot(C2<R>* v, C2<R> f, const C2<R>* __restrict__ T) {
+  if (T) {
+#pragma unroll
+    for (int r = 0; r < 16; ++r)
+      if (r & (1 << K)) v[r] = cmul(v[r], cmul(f, T[r]));
+  } else {
+#pragma unroll
+    for (int r = 0; r < 16; ++r)
+      if (r & (1 << K)) v[r] = cmul(v[r], f);
+  }
+}
+template <typename R>
+__device__ __forceinline__ void apply_cp_run(C2<R>* v, const TileOp<R>* __restrict__ opp, uint64_t ctx, int lw,
+                                             const C2<R>* U, const C2<R>* W, const C2<R>* __restrict__ tabs) {
+  // RunHeader, read as words: n_s, n_f[0] | n_f[1], n_f[2] | n_f[3], ubase | umask, tmask, - | toff | wbase, wmask, slot
+  static_assert(offsetof(RunHeader, n_f) == 2 && offsetof(RunHeader, ubase) == 10 && offsetof(RunHeader, umask) == 12 &&
+                offsetof(RunHeader, tmask) == 13 && offsetof(RunHeader, toff) == 16 && offsetof(RunHeader, wbase) == 20 &&
+                offsetof(RunHeader, wmask) == 22 && offsetof(RunHeader, slot) == 23 && offsetof(TileOp<R>, m0) == 16);
+  const uint4 w0 = *reinterpret_cast<const uint4*>(&opp->m0[0]);
+  const uint2 w1 = *reinterpret_cast<const uint2*>(reinterpret_cast<const unsigned char*>(&opp->m0[0]) + 16);
+  struct {
+    uint32_t n_s, n_f[4], ubase, umask, tmask, toff, wbase, wmask, slot;
+  } h = {w0.x & 0xffffu, {w0.x >> 16, w0.y & 0xffffu, w0.y >> 16, w0.z & 0xffffu}, w0.z >> 16, w0.w & 0xffu,
+         (w0.w >> 8) & 0xffu, w1.x, w1.y & 0xffffu, (w1.y >> 16) & 0xffu, w1.y >> 24};
+  const RunEntry<R>* __restrict__ e = reinterpret_cast<const RunEntry<R>*>(opp + 1);
+  const C2<R>* __restrict__ T = tabs + h.toff;
+  const C2<R> one{R(1), R(0)};
+  if (h.slot) {
+    const int k = (int)h.slot - 1;
+    const int n_f = (int)(h.n_f[0] + h.n_f[1] + h.n_f[2] + h.n_f[3]);   // (only slot k's list is there)
+    C2<R> f = one;
+    if (n_f) f = run_entries(one, e, n_f, ctx);
+    if (h.umask) f = cmul(f, U[h.ubase]);
+    if (h.tmask & 31) {
+      f = cmul(f, T[lw]);
+      T += kRunTable;
+    }
+    if (!(h.tmask & 32)) T = nullptr;
+    switch (k) {
+      case 0: run_in_slot<0>(v, f, T); break;
+      case 1: run_in_slot<1>(v, f, T); break;
+      case 2: run_in_slot<2>(v, f, T); break;
+      default: run_in_slot<3>(v, f, T); break;
+    }
+    return;
+  }
+  C2<R> s = one;
+  if (h.wmask) {
+    const C2<R>* w = W + h.wbase;
+    const uint32_t bits = ((uint32_t)lw & 31u) | ((uint32_t)lw >> 5) << kLaneBits;   // lane, then warp bits
+    for (uint32_t m = h.wmask; m; m &= m - 1) s = cmul(s, csel((bits & m & (0u - m)) != 0, *w++, one));
+  } else {
+    for (int i = 0; i < (int)h.n_s; ++i) {
+      const RunEntry<R> x = e[i];
+      s = cmul(s, csel(((ctx >> x.pa) & (ctx >> x.pb) & 1ull) != 0, x.p, one));
+    }
+  }
+  e += h.n_s;
+  int u = (int)h.ubase;
+  if (h.umask & 1) s = cmul(s, U[u++]);
+  if (h.tmask & 1) {
+    s = cmul(s, T[lw]);
+    T += kRunTable;
+  }
+  if (!((h.umask | h.tmask) & 30) && !(h.n_f[0] | h.n_f[1] | h.n_f[2] | h.n_f[3])) {
+#pragma unroll
+    for (int r = 0; r < 16; ++r) v[r] = cmul(v[r], s);
+  } else {
+    C2<R> f[kRegBits];
+#pragma unroll
+    for (int k = 0; k < kRegBits; ++k) {
+      f[k] = run_entries(one, e, h.n_f[k], ctx);
+      e += h.n_f[k];
+      if (h.umask & (2 << k)) f[k] = cmul(f[k], U[u++]);
+      if (h.tmask & (2 << k)) {
+        f[k] = cmul(f[k], T[lw]);
+        T += kRunTable;
+      }
+    }
+    // the products over slots 0 and 1, then over 2 and 3
+    const C2<R> lo[4] = {s, cmul(s, f[0]), cmul(s, f[1]), cmul(cmul(s, f[0]), f[1])};
+    const C2<R> f23 = cmul(f[2], f[3]);
+#pragma unroll
+    for (int r = 0; r < 16; ++r) {
+      C2<R> d = lo[r & 3];
+      if (r >= 4) d = cmul(d, r < 8 ? f[2] : (r < 12 ? f[3] : f23));
+      v[r] = cmul(v[r], d);
+    }
+  }
+  if (h.tmask & 32) {
+#pragma unroll
+    for (int r = 0; r < 16; ++r) v[r] = cmul(v[r], T[r]);
+  }
+}
+
 // G2: the pass holds dense two-qubit ops; RUNS: it holds packed diagonal runs
 // (TK_RUN).  Each combination is its own instantiation, so that a pass without
 // them keeps the leaner code and register allocation.
+// FP32: three CTAs on an SM, 80 registers each (with two, 7 % slower); only the leanest has to be told.
 template <typename R, bool G2, bool RUNS>
-__global__ void __launch_bounds__(kTileThreads)
+__global__ void __launch_bounds__(kTileThreads, sizeof(R) == 4 && !G2 && !RUNS ? 3 : 0)
     tile_pass_kernel(C2<R>* __restrict__ psi, const __grid_constant__ TileParams<R> P) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C2<R>* sm = reinterpret_cast<C2<R>*>(smem_raw);
@@ -459,7 +632,7 @@ __global__ void __launch_bounds__(kTileThreads)
 
   __shared__ uint8_t s_pos[kTileBits];
   __shared__ uint64_t s_base;
-  __shared__ C2<R> s_U[RUNS ? kMaxRunJobs : 1];   // the CTA's run-job factors
+  __shared__ C2<R> s_U[RUNS ? 2 * kMaxRunJobs : 1];   // the CTA's factors of jobs, then of thread jobs
   if (tid == 0) {
     const int n_nt = P.pass.n_nt;
     uint64_t base = 0;
@@ -468,21 +641,24 @@ __global__ void __launch_bounds__(kTileThreads)
   }
   if (tid < kTileBits) s_pos[tid] = P.pass.pos[tid];
   if constexpr (RUNS) {
-    // one job per thread: the product of its entries' phases at this tile (bits
-    // below kCtxOne are tile bits, kCtxOne the constant 1)
-    if (tid < P.n_jobs) {
+    // one job per warp, an entry per lane: the product of its entries' phases at this
+    // tile (bits below kCtxOne are tile bits, kCtxOne the constant 1)
+    const uint64_t tctx = tile | (1ull << kCtxOne);
+    const C2<R> one{R(1), R(0)};
+    for (int j = warp; j < P.n_jobs + P.n_tjobs; j += kTileThreads / 32) {
+      const bool tj = j >= P.n_jobs;
       RunJob jb;
-      memcpy(&jb, P.jobs + sizeof(RunJob) * tid, sizeof(jb));
-      const uint64_t tctx = tile | (1ull << kCtxOne);
+      memcpy(&jb, tj ? P.tjobs + sizeof(RunJob) * (j - P.n_jobs) : P.jobs + sizeof(RunJob) * j, sizeof(jb));
       const RunEntry<R>* __restrict__ e = reinterpret_cast<const RunEntry<R>*>(P.ops + jb.op + 1) + jb.first;
-      const C2<R> one{R(1), R(0)};
       C2<R> u = one;
-      for (int i = 0; i < jb.count; ++i) {
+      for (int i = lane; i < jb.count; i += 32) {
         const RunEntry<R> x = e[i];
         const uint64_t b = jb.scalar ? ((tctx >> x.pa) & (tctx >> x.pb)) : (tctx >> x.pa);
         u = cmul(u, csel((b & 1ull) != 0, x.p, one));
       }
-      s_U[tid] = u;
+#pragma unroll
+      for (int m = 16; m > 0; m >>= 1) u = cmul(u, shfl_xor_c(u, m));
+      if (lane == 0) s_U[tj ? kMaxRunJobs + (j - P.n_jobs) : j] = u;
     }
   }
   __syncthreads();
@@ -555,7 +731,12 @@ __global__ void __launch_bounds__(kTileThreads)
     }
     for (int o = cur.op_begin; o < cur.op_end;) {
       const uint8_t k0 = ops[o].kind;
-      if (k0 != TK_DIAG && k0 != TK_CP && !(RUNS && k0 == TK_RUN)) {
+      if (RUNS && k0 == TK_RUN) {
+        apply_cp_run<R>(v, ops + o, ctx, tid, s_U, s_U + kMaxRunJobs, P.tabs);
+        o += 1 + ops[o].slot;   // the header and its entry slots
+        continue;
+      }
+      if (k0 != TK_DIAG && k0 != TK_CP) {
         apply_tile_op<R, G2>(v, ops + o, tile, lane, warp);
         o += (G2 && k0 == TK_G2) ? 2 : 1;   // a dense two-qubit op spans two entries
         continue;
@@ -564,18 +745,11 @@ __global__ void __launch_bounds__(kTileThreads)
       dr.reset();
       uint4 hdr = *reinterpret_cast<const uint4*>(ops + o);
       do {
-        const uint32_t kind = hdr.x & 0xffu;
-        if (RUNS && kind == TK_RUN) {
-          dr.add_run(v, ops + o, ctx, tid, s_U, P.tabs);
-          o += 1 + (int)((hdr.x >> 8) & 0xffu);   // the header and its entry slots
-        } else {
-          if (kind == TK_CP) dr.add_cp(v, ops + o, hdr, ctx);
-          else dr.add(v, ops + o, tile, lane, warp);
-          ++o;
-        }
-        if (o >= cur.op_end) break;
+        if ((hdr.x & 0xffu) == TK_CP) dr.add_cp(v, ops + o, hdr, ctx);
+        else dr.add(v, ops + o, tile, lane, warp);
+        if (++o >= cur.op_end) break;
         hdr = *reinterpret_cast<const uint4*>(ops + o);
-      } while ((hdr.x & 0xffu) == TK_DIAG || (hdr.x & 0xffu) == TK_CP || (RUNS && (hdr.x & 0xffu) == TK_RUN));
+      } while ((hdr.x & 0xffu) == TK_DIAG || (hdr.x & 0xffu) == TK_CP);
       dr.flush(v);
     }
   }
@@ -700,8 +874,8 @@ __device__ __forceinline__ void apply_run(C2<R>* vp, C2<R>* vl, const TileOp<R>*
       default: reg_cross<3>(vp, vl, s); break;
     }
     s.add_to(dst, lane);
-    apply_tile_op<R, false>(vp, opp, tile, lane, warp);
-    apply_tile_op<R, false>(vl, opp, tile, lane, warp);
+    apply_tile_op<R, false, false>(vp, opp, tile, lane, warp);
+    apply_tile_op<R, false, false>(vl, opp, tile, lane, warp);
     return;
   }
   const int mask = 1 << opp->slot;
@@ -854,8 +1028,8 @@ __global__ void __launch_bounds__(kTileThreads, sizeof(R) == 4 ? 2 : 1)
         continue;
       }
       if (op->kind != TK_DIAG) {
-        apply_tile_op<R, G2>(vp, op, tile, lane, warp);
-        apply_tile_op<R, G2>(vl, op, tile, lane, warp);
+        apply_tile_op<R, G2, false>(vp, op, tile, lane, warp);
+        apply_tile_op<R, G2, false>(vl, op, tile, lane, warp);
         o += (G2 && op->kind == TK_G2) ? 2 : 1;   // a dense two-qubit op spans two entries
         continue;
       }

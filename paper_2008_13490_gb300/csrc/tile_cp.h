@@ -26,7 +26,10 @@ constexpr int kCtxOne = 47, kCtxLane = 48, kCtxWarp = 56;
 //   register x register      -> table RR over the 16 register indices: into v
 //   tile x tile              -> one factor of the scalar per CTA (a job)
 //   register slot k x tile   -> one factor of f_k[1] per CTA (a job)
-//   tile x thread            -> entries each thread applies (n_s, the residual)
+//   tile x thread            -> the residual entries (n_s, ordered by thread bit): one factor
+//                               per CTA and thread bit (a thread job), multiplied into the
+//                               scalar of the threads where the bit is 1; the entries
+//                               themselves where the jobs do not fit
 // The tables do not depend on the tile: the host builds them (FP64 products,
 // rounded once) into the pass's table buffer.  A job's product is formed once per
 // CTA in the kernel's prologue from its entries.  Entries follow the header in
@@ -39,6 +42,9 @@ struct RunHeader {
   uint8_t umask;       // jobs present: bit 0 scalar, bit 1 + k slot k
   uint8_t tmask;       // tables present: bit 0 S, bit 1 + k N_k, bit 5 RR
   uint32_t toff;       // first table entry (complex index into the pass's table buffer)
+  uint16_t wbase;      // first factor of the run's thread jobs
+  uint8_t wmask;       // thread jobs present (then they stand for the n_s entries): lane bits 0..4, warp bits 5..7
+  uint8_t slot;        // 1 + k: every op has a bit in register slot k (no scalar, no other slot); else 0
 };
 constexpr uint8_t TK_RUN = 6;
 template <typename R>
@@ -55,7 +61,7 @@ struct RunJob {
   uint16_t op, first, count;
   uint8_t scalar, pad;
 };
-constexpr int kMaxRunJobs = 64;
+constexpr int kMaxRunJobs = 64;   // of either sort per pass (thread jobs: pa the tile bit, pb the thread bit)
 constexpr int kRunTable = 1 << (kLaneBits + kWarpBits);   // (lane, warp) entries of S and N_k
 
 // The kernel-parameter image of one forward tile pass (ops in their TK_CP / TK_RUN
