@@ -10,7 +10,7 @@
 //  plain_*_kernel     one launch per gate, the pair/quad update of the thesis's
 //                     four-component loops (Eq. (psioft4componentupdates)) with
 //                     the bit-insert index of its reduced loop, 64-bit indices.
-//  small_state_kernel whole state in one CTA's shared memory (n < 12).
+//  small_state_kernel whole state in the registers of one CTA or a cluster (n < 12).
 //  remap_kernel       permutes bit positions inside a 12-bit tile (in place).
 //  probs / marginal / loglik / reduce: Born rule p_J = |a_J|^2 with fp64
 //                     accumulation of the sums.
@@ -1144,16 +1144,109 @@ __global__ void plain_g2_kernel(C2<R>* __restrict__ psi, int n, PlainOp<R> op) {
 
 // ------------------------------------------------------------------ small states
 
+// A state below a tile: one amplitude per thread, kept in its register through the circuit, on one
+// CTA or a cluster of CTAs (amplitude J of thread J mod T of CTA J / T, T threads).  An op on a lane
+// bit takes its partner's amplitude by a shuffle, on a warp bit through shared memory, on a CTA bit
+// from the other CTA's shared memory.  The ops are staged in shared memory.  Each kind of exchange
+// writes two buffers in turn: who writes one again has passed the barrier of the exchange in
+// between, which every reader reaches after it has used what it read.
+//
+// FP64 is bound by the FP64 pipe of the SMs it runs on, so it takes 128 threads on each of as many
+// as 8 SMs (20 layers of Haar gates and CNOTs, kernel alone: 10 qubits 466 -> 95 us, 11 qubits
+// 854 -> 135, against pairs in one SM's shared memory); FP32 by the latency of an op, so it stays on one SM
+// while that holds the state (8 qubits, 47 ops: 34 -> 13.8 us; 11 qubits, 229 ops: 202 -> 72, where
+// an op read its matrix from global memory and its pairs from shared memory, with a barrier each).
+constexpr int kSmallOps = 256;   // ops staged at a time
+
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ void cluster_barrier() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
 template <typename R>
-__global__ void __launch_bounds__(256)
-    small_state_kernel(C2<R>* __restrict__ psi, int n, const PlainOp<R>* __restrict__ ops, int nops) {
+__device__ __forceinline__ C2<R> ld_cluster(const C2<R>* p, uint32_t rank) {
+  uint32_t a = (uint32_t)__cvta_generic_to_shared(p);
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(a), "r"(rank));
+  C2<R> v;
+  if constexpr (sizeof(R) == 8)
+    asm volatile("ld.shared::cluster.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "r"(a) : "memory");
+  else
+    asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(a) : "memory");
+  return v;
+}
+
+template <typename R>
+__global__ void __launch_bounds__(sizeof(R) == 4 ? 1024 : 256)
+    small_state_kernel(C2<R>* __restrict__ psi, int n, int tbits, const PlainOp<R>* __restrict__ ops, int nops) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  C2<R>* sm = reinterpret_cast<C2<R>*>(smem_raw);
-  const int N = 1 << n;
-  for (int J = threadIdx.x; J < N; J += blockDim.x) sm[J] = psi[J];
-  __syncthreads();
-  small_apply_ops(sm, n, ops, nops);
-  for (int J = threadIdx.x; J < N; J += blockDim.x) psi[J] = sm[J];
+  const uint32_t T = 1u << tbits, tid = threadIdx.x;
+  C2<R>* xb = reinterpret_cast<C2<R>*>(smem_raw);                 // exchanges in the CTA: 2 x blockDim.x
+  C2<R>* cb = xb + 2 * blockDim.x;                                // in the cluster: 2 x blockDim.x
+  PlainOp<R>* sop = reinterpret_cast<PlainOp<R>*>(cb + 2 * blockDim.x);
+  const bool clustered = n > tbits;
+  const uint32_t rank = clustered ? cluster_rank() : 0;
+  const uint32_t J = (rank << tbits) | tid;
+  const bool live = tid < T;                                      // (fewer than 32 amplitudes)
+  C2<R> v{R(0), R(0)};
+  if (live) v = psi[J];
+  uint32_t xi = 0, ci = 0;                                        // the next buffer of either kind
+  // after this the amplitude of J ^ mask is at buf[(tid ^ mask) mod T] of CTA rank ^ (mask / T)
+  auto publish = [&](uint32_t mask) -> const C2<R>* {
+    if (mask >= T) {
+      C2<R>* buf = cb + ci * blockDim.x;
+      ci ^= 1;
+      buf[tid] = v;
+      cluster_barrier();
+      return buf;
+    }
+    C2<R>* buf = xb + xi * blockDim.x;
+    xi ^= 1;
+    buf[tid] = v;
+    __syncthreads();
+    return buf;
+  };
+  auto read = [&](const C2<R>* buf, uint32_t j) -> C2<R> {        // the amplitude of index j
+    const uint32_t r = j >> tbits;
+    const C2<R>* p = buf + (j & (T - 1));
+    return r == rank ? *p : ld_cluster(p, r);
+  };
+  for (int k0 = 0; k0 < nops; k0 += kSmallOps) {
+    const int cnt = min(kSmallOps, nops - k0);
+    if (k0) __syncthreads();                                      // the last ones have been read
+    const uint4* src = reinterpret_cast<const uint4*>(ops + k0);
+    uint4* dst = reinterpret_cast<uint4*>(sop);
+    for (uint32_t i = tid; i < cnt * (uint32_t)(sizeof(PlainOp<R>) / 16); i += blockDim.x) dst[i] = src[i];
+    __syncthreads();
+    for (int k = 0; k < cnt; ++k) {
+      const PlainOp<R>* op = sop + k;
+      const int type = op->type;
+      if (type == F_G1 || type == F_G1C) {
+        const uint32_t mask = 1u << op->t;
+        const C2<R>* m = op->m;
+        if (type == F_G1C && ((J >> op->c) & 1u)) m += 4;
+        const C2<R> q = mask < 32u ? shfl_xor_c(v, (int)mask) : read(publish(mask), J ^ mask);
+        const bool up = (J & mask) != 0;
+        if (up) m += 2;
+        v = cfma2(m[0], csel(up, q, v), m[1], csel(up, v, q));
+      } else if (type == F_D) {
+        const uint32_t ba = (J >> op->a) & 1u;
+        v = cmul(v, op->m[op->b >= 0 ? ba * 2 + ((J >> op->b) & 1u) : ba]);
+      } else {
+        const uint32_t ma = 1u << op->a, mb = 1u << op->b, base = J & ~(ma | mb);
+        const C2<R>* buf = publish(ma | mb);
+        const C2<R>* m = op->m + 4 * (((J & ma) ? 2 : 0) + ((J & mb) ? 1 : 0));
+        // (a thread beyond the state, where there are fewer amplitudes than lanes, works on its own zeros)
+        const C2<R> y0 = cfma2(m[0], live ? read(buf, base) : v, m[1], live ? read(buf, base | mb) : v);
+        const C2<R> y1 = cfma2(m[2], live ? read(buf, base | ma) : v, m[3], live ? read(buf, base | ma | mb) : v);
+        v = C2<R>{y0.x + y1.x, y0.y + y1.y};
+      }
+    }
+  }
+  if (live) psi[J] = v;
+  if (clustered) cluster_barrier();                               // nobody reads this CTA's buffers any more
 }
 
 // ------------------------------------------------------------------ remap
@@ -1715,21 +1808,33 @@ qs_status launch_plain_op(State* st, const void* op_host, int /*type*/) {
   return plain_launch_t<double>(st, *(const PlainOp<double>*)op_host);
 }
 
-qs_status launch_small(State* st, const void* ops_dev, int nops) {
-  const size_t smem = st->amp_bytes << st->n;
-  if (st->prec == QS_C64) {
-    qs_status s = set_smem(small_state_kernel<float>, smem);
-    if (s != QS_OK) return s;
-    small_state_kernel<float><<<1, 256, smem, st->stream>>>((C2<float>*)st->data, st->n,
-                                                            (const PlainOp<float>*)ops_dev, nops);
-  } else {
-    qs_status s = set_smem(small_state_kernel<double>, smem);
-    if (s != QS_OK) return s;
-    small_state_kernel<double><<<1, 256, smem, st->stream>>>((C2<double>*)st->data, st->n,
-                                                             (const PlainOp<double>*)ops_dev, nops);
-  }
-  QS_CUDA(cudaGetLastError());
+template <typename R>
+static qs_status small_launch_t(State* st, const void* ops_dev, int nops) {
+  const int n = st->n;
+  // FP64: 128 threads per SM (one warp on each of its FP64 pipes) on at most 8 SMs, the largest
+  // portable cluster; FP32: one SM up to 1024 amplitudes
+  const int tbits = sizeof(R) == 8 ? std::max(std::min(n, 7), n - 3) : std::min(n, 10);
+  const unsigned threads = 1u << std::max(tbits, 5);
+  const size_t smem = 4 * threads * sizeof(C2<R>) + sizeof(PlainOp<R>) * (size_t)std::min(nops, kSmallOps);
+  qs_status s = set_smem(small_state_kernel<R>, smem);
+  if (s != QS_OK) return s;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(1u << (n - tbits));
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st->stream;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = cfg.gridDim.x;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  QS_CUDA(cudaLaunchKernelEx(&cfg, small_state_kernel<R>, (C2<R>*)st->data, n, tbits, (const PlainOp<R>*)ops_dev, nops));
   return QS_OK;
+}
+
+qs_status launch_small(State* st, const void* ops_dev, int nops) {
+  return st->prec == QS_C64 ? small_launch_t<float>(st, ops_dev, nops) : small_launch_t<double>(st, ops_dev, nops);
 }
 
 qs_status launch_remap(State* st, const RemapDesc& d) {
