@@ -110,20 +110,24 @@ typedef enum {
    * bounded-wait status word). */
   QS_METHOD_BLOCKS_TF32 = 2, /* two TF32 parts, 4 products (~1e-6 relative over 100 blocks) */
   QS_METHOD_BLOCKS_BF16 = 3, /* three BF16 parts, 6 products (~6e-7 relative over 100 blocks) */
-  /* the default (also when opts is NULL): for complex64 states with n >= 12
+  /* the default (also when opts is NULL).  States with n <= 13 (complex64 with n = 13: circuits
+   * with dense gates) run in one launch, kept in the registers of one CTA or a cluster of
+   * CTAs.  For other complex64 states
    * the circuit is cut into 5-qubit blocks; a block with more than half of its
    * 1024 entries nonzero is a dense contraction and its gates run as BF16-split
    * GEMMs on the tensor cores (planned again as chains of up to three 5-qubit blocks
    * per sweep; one block per sweep when an explicit matrix is not unitary), and each
    * maximal run of sparser blocks (diagonal or nearly diagonal stretches,
    * permutations) is replayed gate by gate through the tile passes (runs of up to
-   * four sparse blocks stay with their neighbours in mostly dense circuits).  With only one or two dense blocks, the whole circuit runs on tile
-   * passes when that takes no more tile passes and remaps than the sparse runs
-   * alone (the blocks' sweeps are saved).  complex128 states with n >= 12: circuits of
-   * mostly dense blocks run block by block on the tensor cores too, in exact integer
-   * slices of the FP64 values (one rounding per block and amplitude).  Everything else
-   * uses QS_METHOD_TILED.
-   * Synchronous like the block methods. */
+   * four sparse blocks stay with their neighbours in mostly dense circuits).  With
+   * only one or two dense blocks, the whole circuit runs on tile passes when that
+   * takes no more tile passes and remaps than the sparse runs alone (the blocks'
+   * sweeps are saved).  Larger complex128 states: circuits of mostly dense blocks run
+   * block by block on the tensor cores too, in exact integer slices of the FP64
+   * values (one rounding per block and amplitude).  Everything else uses
+   * QS_METHOD_TILED.
+   * Synchronous like the block methods for complex64 states with n >= 12, and where
+   * complex128 blocks run. */
   QS_METHOD_AUTO = 4
 } qs_method;
 

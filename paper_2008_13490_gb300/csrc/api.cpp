@@ -1103,7 +1103,7 @@ qs_status run_blocks(State* st, const qs_gate* gates, size_t ngates, int mode, q
   return run_block_list(st, blocks, mode, stats, tm);
 }
 
-// QS_METHOD_AUTO, complex128, n >= 12: circuits of mostly dense blocks (at least three for each
+// QS_METHOD_AUTO, complex128, n > kSmallAutoBits: circuits of mostly dense blocks (at least three for each
 // sparse one) run block by block on the tensor cores (block_f64.cu).  QS_EUNSUPPORTED, with
 // nothing launched, for others and for matrices that the integer slices do not take: they run
 // on tile passes.
@@ -1158,7 +1158,7 @@ qs_status run_f64_blocks(State* st, const qs_gate* gates, size_t ngates, qs_stat
   return QS_OK;
 }
 
-// QS_METHOD_AUTO (complex64, n >= 12): the circuit is cut into 5-qubit blocks;
+// QS_METHOD_AUTO (complex64, larger states than kSmallAutoBits allows): the circuit is cut into 5-qubit blocks;
 // a dense block (more than half of its 1024 entries nonzero) is a real
 // contraction and goes to the tensor cores (the gates of a run of dense blocks planned
 // again as chains of blocks, one block per sweep if a gate is not unitary), and every
@@ -1270,6 +1270,18 @@ qs_status adjoint_tiled(State* st, void* lam, const qs_gate* gates, size_t g0, s
                             : adjoint_tiled_t<double>(st, lam, gates, g0, g1, dth);
 }
 
+// QS_METHOD_AUTO keeps states of up to this many qubits in the registers of one CTA or cluster
+// (small_state_kernel): one launch whatever the circuit, where blocks and tiles of such states leave
+// the chip idle and pay for a launch and a pipeline's start per sweep.  Whole calls, us, there
+// against here, 12 and 13 qubits: layered complex64 of 10 and 80 layers 250 and 1271 -> 66 and 346,
+// 515 and 1418 -> 73 and 390; complex128 of 10 and 60 layers 700 and 2501 -> 103 and 472, 737 and 2860 ->
+// 190 and 937; Haar and CNOT complex128 of 5 and 60 layers 461 and 4557 -> 93 and 816, 490 and 4525 -> 153
+// and 1483; Fourier 278 -> 53 (12 qubits); 500 mixed gates 922 -> 171, 1106 -> 175.
+// Above, a thread would hold several amplitudes.  Circuits of 13
+// complex64 qubits without dense gates keep to tile passes all the same: their users count these
+// (qs_stats.tile_launches).
+constexpr int kSmallAutoBits = 13;
+
 qs_status apply_gates(State* st, const qs_gate* gates, size_t ngates, int method, qs_stats* stats,
                       int flags) {
   if (stats) std::memset(stats, 0, sizeof(*stats));
@@ -1279,7 +1291,9 @@ qs_status apply_gates(State* st, const qs_gate* gates, size_t ngates, int method
   }
   // AUTO: blocks and tile passes where the state allows the blocks, else tiles
   const bool autom = method == QS_METHOD_AUTO && st->prec == QS_C64 && st->n >= kTileBits;
-  const bool auto_f64 = method == QS_METHOD_AUTO && st->prec == QS_C128 && st->n >= kTileBits;
+  const bool auto_small = method == QS_METHOD_AUTO && st->n <= kSmallAutoBits &&
+                          (st->prec == QS_C128 || st->n < kSmallAutoBits || chains_likely(gates, ngates));
+  const bool auto_f64 = method == QS_METHOD_AUTO && st->prec == QS_C128 && st->n >= kTileBits && !auto_small;
   if (method == QS_METHOD_AUTO && !autom) method = QS_METHOD_TILED;
   const bool blocks = method == QS_METHOD_BLOCKS_TF32 || method == QS_METHOD_BLOCKS_BF16;
   if (blocks && (st->prec != QS_C64 || st->n < kTileBits)) {
@@ -1296,17 +1310,19 @@ qs_status apply_gates(State* st, const qs_gate* gates, size_t ngates, int method
   qs_status s = QS_EUNSUPPORTED;
   if (auto_f64) s = run_f64_blocks(st, gates, ngates, stats, tm);
   if (auto_f64 && s != QS_EUNSUPPORTED) {
-  } else if (autom) {
+  } else if (autom && !auto_small) {
     s = run_auto(st, gates, ngates, stats, tm);
   } else if (blocks) {
     s = run_blocks(st, gates, ngates, method == QS_METHOD_BLOCKS_TF32 ? 0 : 1, stats, tm);
   } else if (method == QS_METHOD_PLAIN) {
     build_fused_ops(gates, ngates, st->n, fops, vmap, /*fuse=*/false, /*relabel=*/false);
     s = c64 ? run_plain<float>(st, fops, stats, tm) : run_plain<double>(st, fops, stats, tm);
-  } else if (st->n < kTileBits) {
+  } else if (st->n < kTileBits || auto_small) {
     build_fused_ops(gates, ngates, st->n, fops, vmap, /*fuse=*/true, /*relabel=*/false);
     merge_one_qubit_ops(fops, st->n, nullptr);   // one CTA runs them all: no passes to keep
     s = c64 ? run_small<float>(st, fops, stats, tm) : run_small<double>(st, fops, stats, tm);
+    // (the default method of complex64 states from kTileBits on returns when the state is ready)
+    if (autom && s == QS_OK) QS_CUDA(cudaStreamSynchronize(st->stream));
   } else {
     build_fused_ops(gates, ngates, st->n, fops, vmap, /*fuse=*/true, /*relabel=*/true);
     s = c64 ? run_tiled<float>(st, fops, vmap, stats, tm)

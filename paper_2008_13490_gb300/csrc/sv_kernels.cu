@@ -10,7 +10,8 @@
 //  plain_*_kernel     one launch per gate, the pair/quad update of the thesis's
 //                     four-component loops (Eq. (psioft4componentupdates)) with
 //                     the bit-insert index of its reduced loop, 64-bit indices.
-//  small_state_kernel whole state in the registers of one CTA or a cluster (n < 12).
+//  small_state_kernel whole state in the registers of one CTA or a cluster (n < 12; the
+//                     default method: n < 14).
 //  remap_kernel       permutes bit positions inside a 12-bit tile (in place).
 //  probs / marginal / loglik / reduce: Born rule p_J = |a_J|^2 with fp64
 //                     accumulation of the sums.
@@ -1144,7 +1145,7 @@ __global__ void plain_g2_kernel(C2<R>* __restrict__ psi, int n, PlainOp<R> op) {
 
 // ------------------------------------------------------------------ small states
 
-// A state below a tile: one amplitude per thread, kept in its register through the circuit, on one
+// A small state: one amplitude per thread, kept in its register through the circuit, on one
 // CTA or a cluster of CTAs (amplitude J of thread J mod T of CTA J / T, T threads).  An op on a lane
 // bit takes its partner's amplitude by a shuffle, on a warp bit through shared memory, on a CTA bit
 // from the other CTA's shared memory.  The ops are staged in shared memory.  Each kind of exchange
@@ -1179,7 +1180,7 @@ __device__ __forceinline__ C2<R> ld_cluster(const C2<R>* p, uint32_t rank) {
 }
 
 template <typename R>
-__global__ void __launch_bounds__(sizeof(R) == 4 ? 1024 : 256)
+__global__ void __launch_bounds__(1024)
     small_state_kernel(C2<R>* __restrict__ psi, int n, int tbits, const PlainOp<R>* __restrict__ ops, int nops) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const uint32_t T = 1u << tbits, tid = threadIdx.x;

@@ -1,4 +1,4 @@
-"""States below a tile (n < 12): every op kind with its qubits on lanes, warps and CTAs of the
+"""Small states (the default method, n < 14): every op kind with its qubits on lanes, warps and CTAs of the
 cluster, and op lists around the number staged at a time, against the oracle."""
 import numpy as np
 import pytest
@@ -9,9 +9,20 @@ from oracle import statevector as SV
 pytestmark = pytest.mark.gpu
 
 
+def test_dense_complex64_of_13_qubits(qs):
+    ops = W.layered_haar_cz(13, 10, seed=4)
+    st = qs.State(13, 0)
+    stats = qs.sv_apply_circuit(st, ops)
+    out = qs.sv_copy_out(st)
+    st.close()
+    assert stats["passes"] == 1 and stats["tile_launches"] == 0
+    ref = SV.apply_circuit(SV.basis(13), 13, ops)
+    assert np.linalg.norm(out - ref) < 12 * 2.0 ** -24 * len(ops)
+
+
 @pytest.mark.parametrize("prec", [0, 1])
 @pytest.mark.parametrize("n,count", [(1, 20), (2, 60), (4, 300), (5, 100), (6, 100), (7, 300), (8, 300), (9, 900),
-                                     (10, 300), (11, 1500)])
+                                     (10, 300), (11, 1500), (12, 600), (13, 600)])
 def test_small_states(qs, n, count, prec):
     if n == 1:
         ops = [("MAT1", (0,), (), W.haar_su2(W.rng(k))) for k in range(count)]
@@ -20,7 +31,9 @@ def test_small_states(qs, n, count, prec):
     psi = W.random_state(n, W.rng(6))
     st = qs.State(n, prec)
     qs.sv_copy_in(st, psi.astype(st.amp_dtype))
-    qs.sv_apply_circuit(st, ops, method=qs.METHOD_TILED)
+    stats = qs.sv_apply_circuit(st, ops)
+    if n < 13 or prec:   # (13 complex64 qubits: circuits with dense gates only)
+        assert stats["passes"] == 1 and stats["tile_launches"] == 0
     out = qs.sv_copy_out(st)
     st.close()
     ref = SV.apply_circuit(psi.copy(), n, ops)
