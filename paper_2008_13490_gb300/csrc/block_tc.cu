@@ -456,7 +456,6 @@ __global__ void __launch_bounds__(kPipeThreads, 1)
           x[16 + j] = raw[e ^ ec16];
         }
       }
-      mbar_arrive(&rempty[s]);   // the row is in registers: raw stage s may be refilled
       float nrm[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
       for (int j = 0; j < 32; ++j) {
@@ -465,6 +464,9 @@ __global__ void __launch_bounds__(kPipeThreads, 1)
       }
       // keep the norm here: sunk to its store it would keep a copy of the row alive
       asm volatile("" : "+f"(nrm[0]), "+f"(nrm[1]), "+f"(nrm[2]), "+f"(nrm[3]));
+      // raw stage s may be refilled: the row has been used (an arrival straight after the loads
+      // can be seen before loads that wait for a bank have read)
+      mbar_arrive(&rempty[s]);
       // slot j <- column 16 h + j
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
