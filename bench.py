@@ -5,11 +5,11 @@ Workload (the 30-qubit configuration): n = 30 qubits, complex64 (8 GiB
 state), 40 layers of Haar-random SU(2) on every qubit plus brickwork CZ
 (seed 2001) = 1780 gates, started from |0...0>, followed by the Born-rule
 probabilities (4 GiB fp32) and their fp64 norm.  One step = one such circuit,
-by default through the library's default method (QS_METHOD_AUTO: dense 5-qubit
-blocks on the tcgen05 tensor cores with the BF16 three-part split and FP32
-accumulation, sparse stretches on tile passes; for this circuit 93 of the 100
-blocks are dense and the gates of the other 7 take 3 tile passes; --method
-selects another), the tiled FP32 SIMT path reported as a row of the same line.
+by default through the library's default method (QS_METHOD_AUTO: chains of up to
+three dense 5-qubit blocks per sweep on the tcgen05 tensor cores with the BF16
+three-part split and FP32 accumulation, sparse stretches on tile passes; this
+circuit takes 37 sweeps of 109 blocks and no tile pass; --method selects
+another), the tiled FP32 SIMT path reported as a row of the same line.
 
 metric: reported in "gates/s" = gates of the circuit applied to the
 full 2^30-amplitude state per second (the real HBM sweeps per second are in
@@ -95,9 +95,9 @@ def alu_peaks(qs, torch):
 
 
 METHOD_NOTE = {
-    "auto": "the library's default: the circuit cut into 5-qubit blocks, dense blocks as BF16-split "
-            "GEMMs on tcgen05 tensor cores (FP32 accumulation, per-row norm correction), runs of "
-            "sparse blocks replayed through 12-qubit shared-memory tile passes",
+    "auto": "the library's default: the circuit cut into 5-qubit blocks, chains of up to three dense "
+            "blocks per sweep as BF16-split GEMMs on tcgen05 tensor cores (FP32 accumulation, norm "
+            "correction per sweep), runs of sparse blocks replayed through 12-qubit shared-memory tile passes",
     "blocks_bf16": "5-qubit fused blocks on tcgen05 tensor cores, BF16 three-part split products, "
                    "FP32 accumulation, per-row norm correction",
     "blocks_tf32": "5-qubit fused blocks on tcgen05 tensor cores, TF32 two-part split products, "
@@ -115,7 +115,6 @@ KERNEL_SOURCES = {
 TRAFFIC_FILES = {
     ("tile", "tiled"): "tile_pass_kernel_traffic_n30_layered_haar_cz.json",
     ("block", "blocks_bf16"): "block_pipe_kernel_bf16_traffic_n30_layered_haar_cz.json",
-    ("block", "auto"): "block_pipe_kernel_bf16_traffic_n30_layered_haar_cz.json",
 }
 
 
@@ -500,13 +499,18 @@ def run_ours(args, world, rank, local):
                 "peak": alu["fp32_tflops"],
                 "peak_source": "FP32 FMA peak measured in this run (qs_alu_peak)"}
     elif dominant == "block":
-        # block GEMM: one HBM sweep per launch (its roof; the tensor work, 4 (TF32) or
-        # 6 (BF16) split products of 2^(n+8) flops, is far below the tensor peak)
+        # block GEMMs: one HBM sweep per launch (its roof; the tensor work, 4 (TF32) or
+        # 6 (BF16) split products of 2^(n+8) flops per block, is far below the tensor peak);
+        # the default method applies several blocks per sweep
         per_launch = bytes_per_pass
         tf32 = args.method == "blocks_tf32"   # (the default method uses the BF16 split)
-        roof = {"bound": "hbm", "kernel": "block_pipe_kernel<%s>" % ("TF32" if tf32 else "BF16"),
+        chains = args.method == "auto"
+        blocks = stats["ops_fused"] / max(1, stats["passes"]) if chains and not stats["tile_launches"] else 1
+        roof = {"bound": "hbm",
+                "kernel": "chain_kernel" if chains else "block_pipe_kernel<%s>" % ("TF32" if tf32 else "BF16"),
                 "unit": "GB/s", "peak": peaks["hbm_gbs"], "peak_source": "measured copy bandwidth",
-                "tensor_tflops": block_products(tf32) * 2.0 ** (n + 8) / (avg_ms * 1e-3) / 1e12,
+                "blocks_per_launch": blocks,
+                "tensor_tflops": blocks * block_products(tf32) * 2.0 ** (n + 8) / (avg_ms * 1e-3) / 1e12,
                 "tensor_peak_tflops": alu["tf32_tflops"] if tf32 else peaks["bf16_tflops"],
                 "tensor_peak_source": "TF32: cuBLAS GEMM measured in this run" if tf32
                 else "bf16 burst, MEASURED_PEAKS.json"}
