@@ -791,8 +791,9 @@ __global__ void __launch_bounds__(kTileThreads, sizeof(R) == 4 && !G2 && !RUNS ?
 // through the pass; an op's sums over the tile go to s_term (warp sums, shared-memory
 // atomics), written per tile to partial[tile][sum].
 //
-// The FP32 pipe bounds it (24 qubits, 20 layers of three rotations and CZs: 480 runs).  With a term op and a U^dagger per gate, three of each per run, and the CZs as
-// diagonals of their own the sweep took 40.1 ms, now 9.9 (11 passes, now 8).
+// The FP32 pipe bounds it (24 qubits, 20 layers of three rotations and CZs: 480 runs).  With a
+// term op and a U^dagger per gate, three of each per run, and the CZs as diagonals of their own,
+// the sweep took 40.1 ms in 11 passes; now 10.1 in 8.
 
 // The sums over this thread's amplitudes that an op of a TermRec takes.
 template <typename R>
