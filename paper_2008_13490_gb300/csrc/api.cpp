@@ -1265,6 +1265,61 @@ template void tile_pass_image<float>(const Plan&, const TilePass&, TileParams<fl
 template void tile_pass_image<double>(const Plan&, const TilePass&, TileParams<double>*, std::vector<C2<double>>&);
 
 
+template <typename R>
+qs_status adjoint_small_t(State* st, void* lam, const qs_gate* gates, size_t ng, double* dth) {
+  AdjointOps ad;
+  qs_status s = adjoint_ops(gates, 0, ng, st->n, ad);
+  if (s != QS_OK || ad.ops.empty()) return s;
+  constexpr int kSums = 4096;   // of one launch: bounds the partials
+  struct Part {
+    int op, nop, rec, nrec, nsum;
+  };
+  std::vector<Part> parts{{0, 0, 0, 0, 0}};
+  std::vector<PlainOp<R>> ops;
+  std::vector<TermRec> recs;
+  for (const FOp& o : ad.ops) {
+    PlainOp<R> p = to_plain<R>(o);
+    p.pad[0] = 0;
+    if (o.term >= 0) {
+      TermRec r = ad.recs[(size_t)o.term];
+      if (parts.back().nsum + r.nsum > kSums) parts.push_back({(int)ops.size(), 0, (int)recs.size(), 0, 0});
+      r.sum = parts.back().nsum;
+      p.pad[0] = 1 + r.sum;
+      parts.back().nsum += r.nsum;
+      ++parts.back().nrec;
+      recs.push_back(r);
+    }
+    ops.push_back(p);
+    ++parts.back().nop;
+  }
+  const size_t pbytes = sizeof(double) * (size_t)adjoint_small_warps(st) * kSums;
+  double* partial = (double*)dev_alloc(st, pbytes);
+  if (!partial) {
+    set_error("adjoint partials allocation failed");
+    return QS_ENOMEM;
+  }
+  std::vector<unsigned char> blob;
+  const size_t off_ops = put(blob, ops.data(), ops.size());
+  const size_t off_recs = put(blob, recs.data(), recs.size());
+  const size_t off_pars = put(blob, ad.pars.data(), ad.pars.size());
+  s = upload(st, blob);
+  unsigned char* dev = (unsigned char*)st->opbuf;
+  for (size_t i = 0; i < parts.size() && s == QS_OK; ++i) {
+    const Part& q = parts[i];
+    s = launch_adjoint_small(st, lam, dev + off_ops + sizeof(PlainOp<R>) * (size_t)q.op, q.nop, partial, q.nsum,
+                             (const TermRec*)(dev + off_recs) + q.rec, q.nrec, (const TermPar*)(dev + off_pars), dth);
+  }
+  cudaStreamSynchronize(st->stream);
+  dev_free(st, partial, pbytes);
+  return s;
+}
+
+qs_status adjoint_small(State* st, void* lam, const qs_gate* gates, size_t ng, double* dth) {
+  if (!gates_unitary(gates, ng)) return QS_EUNSUPPORTED;
+  return st->prec == QS_C64 ? adjoint_small_t<float>(st, lam, gates, ng, dth)
+                            : adjoint_small_t<double>(st, lam, gates, ng, dth);
+}
+
 qs_status adjoint_tiled(State* st, void* lam, const qs_gate* gates, size_t g0, size_t g1, double* dth) {
   return st->prec == QS_C64 ? adjoint_tiled_t<float>(st, lam, gates, g0, g1, dth)
                             : adjoint_tiled_t<double>(st, lam, gates, g0, g1, dth);

@@ -10,7 +10,8 @@
 // registers, the U^dagger and derivative terms of all of a pass's gates in one
 // read+write of psi and lambda; dL/dt = 2 Re <lambda_g | G psi_g> with
 // G = (dU/dt) U^dagger, and for a run of one-qubit gates on a qubit all of these
-// from the same four inner products).  Otherwise one kernel per gate computes
+// from the same four inner products).  Smaller states go through the same ops in one launch
+// (adjoint_small_kernel).  With checkpoints, or matrices that are not unitary, one kernel per gate computes
 // psi_{g-1} = U_g^dagger psi_g, the derivative terms (fp64 block partials) and
 // lambda_{g-1} = U_g^dagger lambda_g.
 // Rotation derivatives follow from R(t) = exp(-i t sigma/2)
@@ -374,7 +375,16 @@ qs_status run_grad(State* st, const qs_gate* gates, size_t ng, const double* w, 
       }
     }
   }
-  if (s == QS_OK && !fused) {
+  // smaller states without checkpoints in one launch, else (checkpoints: states stored before each
+  // gate; matrices that are not unitary) a launch per gate
+  bool stepped = !fused;
+  if (s == QS_OK && !fused && !use_ckpt) {
+    QS_CUDA(cudaMemsetAsync(dth, 0, sizeof(double) * 3 * ng, st->stream));
+    s = adjoint_small(st, lam, gates, ng, dth);
+    stepped = s == QS_EUNSUPPORTED;
+    if (stepped) s = QS_OK;
+  }
+  if (s == QS_OK && stepped) {
     for (int k = 0; use_ckpt && k < K && s == QS_OK; ++k) {
       C2<R>* b = (C2<R>*)alloc_state();
       if (!b) {
@@ -384,7 +394,7 @@ qs_status run_grad(State* st, const qs_gate* gates, size_t ng, const double* w, 
       segbuf.push_back(b);
     }
   }
-  if (s == QS_OK && !fused) {
+  if (s == QS_OK && stepped) {
     if (!use_ckpt) {
       for (size_t g = ng; g-- > 0 && s == QS_OK;)
         s = backward_gate<R>(st, (C2<R>*)st->data, lam, gates[g], partials, done, dth + 3 * g, false);

@@ -40,7 +40,7 @@ def _runs(n, g):
 
 
 @pytest.mark.parametrize("prec", [0, 1])
-@pytest.mark.parametrize("n,ckpt", [(12, 0), (13, 20), (15, 0)])
+@pytest.mark.parametrize("n,ckpt", [(2, 0), (4, 0), (6, 7), (7, 0), (8, 0), (10, 0), (11, 0), (12, 0), (13, 20), (15, 0)])
 def test_runs(qs, n, prec, ckpt):
     ops = _runs(n, W.rng(40 + n))
     _check(qs, n, ops, prec, ckpt)
@@ -52,6 +52,18 @@ def test_more_sums_than_a_pass_holds(qs, prec):
     n, g = 12, W.rng(9)
     ops = []
     for layer in range(9):
+        ops += [("RX" if layer % 2 else "RY", (q,), (g.uniform(-3, 3),), None) for q in range(n)]
+        ops += [("CNOT", (a, a + 1), (), None) for a in range(layer % 2, n - 1, 2)]
+        ops += [("H", (0,), (), None), ("H", (n - 1,), (), None)]
+    _check(qs, n, ops, prec, 0)
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+def test_more_sums_than_a_launch_holds(qs, prec):
+    # 1200 runs of 4 sums below a tile: beyond 4096
+    n, g = 6, W.rng(10)
+    ops = []
+    for layer in range(200):
         ops += [("RX" if layer % 2 else "RY", (q,), (g.uniform(-3, 3),), None) for q in range(n)]
         ops += [("CNOT", (a, a + 1), (), None) for a in range(layer % 2, n - 1, 2)]
         ops += [("H", (0,), (), None), ("H", (n - 1,), (), None)]
