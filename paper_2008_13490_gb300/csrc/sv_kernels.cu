@@ -1774,8 +1774,14 @@ __global__ void __launch_bounds__(256)
     loglik_kernel(const C2<R>* __restrict__ psi, const uint32_t* __restrict__ counts, uint64_t N,
                   double* __restrict__ partials, unsigned long long* __restrict__ clamps) {
   constexpr int kBatch = 8;   // loads in flight per thread
+  // a small state takes as many blocks as have a batch for each thread: its logarithm costs more
+  const uint64_t blocks = min((uint64_t)gridDim.x, max(N / (kBatch * blockDim.x), (uint64_t)1));
+  if (blockIdx.x >= blocks) {
+    if (threadIdx.x == 0) partials[blockIdx.x] = 0.0;
+    return;
+  }
   LogProduct l;
-  const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+  const uint64_t stride = blocks * blockDim.x;
   uint64_t J = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
   for (; J + (kBatch - 1) * stride < N; J += kBatch * stride) {
     C2<R> a[kBatch];
@@ -2096,9 +2102,11 @@ qs_status launch_probs(State* st, void* out, int out_fp64, uint64_t mask, double
       ++P.n_rest;
     }
   }
-  // units of lines: about one per warp of the grid
+  // units of lines: about one per warp of the grid, of 16 lines at least while there are 256 units
+  // (each ends in up to 32 atomic additions)
   const int want = 13 - P.n_hi;   // log2(kReduceBlocks * 8 warps)
   P.chunk = P.n_rest - std::max(0, std::min(P.n_rest, want));
+  P.chunk = std::max(P.chunk, std::min({4, P.n_rest, std::max(0, P.n_hi + P.n_rest - 8)}));
   const uint64_t H = 1ull << k;
   QS_CUDA(cudaMemsetAsync(marg_acc, 0, H * sizeof(double), st->stream));
   if (st->prec == QS_C64)
