@@ -95,8 +95,9 @@ struct FOp {
 
 // Converts gates into fused ops.  vmap_out[q] = virtual qubit that holds logical
 // qubit q at the end (SWAPs become relabelings).
-// fuse: merge one-qubit runs and fold diagonals; relabel: SWAPs become
-// relabelings (else they are dense two-qubit ops).
+// fuse: merge one-qubit runs and fold diagonals; relabel: a list for tile passes: SWAPs
+// become relabelings (else they are dense two-qubit ops), and real ops beside runs of
+// phases stay real.
 void build_fused_ops(const qs_gate* gates, size_t ngates, int n, std::vector<FOp>& out,
                      std::vector<int>& vmap_out, bool fuse, bool relabel);
 

@@ -99,10 +99,6 @@ bool fold_into(const FOp& D, FOp& G, bool after) {
   bool t_in = (t == D.a) || (t == D.b);
   if (!t_in) return false;
   int other = (D.b < 0) ? -1 : (t == D.a ? D.b : D.a);
-  // A real op (H, RY, X, CNOT) stays real: it takes half the instructions, and the phase joins a
-  // run of its own kind at less than it would add here (30-qubit Fourier transform: 52.3 ms with
-  // the phase folded in, 46.1 without).
-  if (other >= 0 && (G.type == F_G1 || G.type == F_G1C) && is_real(G) && !is_real(D)) return false;
   if (G.type == F_G1) {
     if (other < 0) {
       cd d0, d1;
@@ -271,6 +267,28 @@ void build_fused_ops(const qs_gate* gates, size_t ngates, int n, std::vector<FOp
       for (int q = 0; q < n; ++q)
         if ((m >> q) & 1) on[q].push_back((int)i);
     }
+    // In a tile pass (relabel) a real op (H, RY, X, CNOT) takes half the instructions of a complex one,
+    // and a phase that meets another on the op's qubit is an entry of their run, which costs less than
+    // the op's becoming complex; a lone phase would be an op of its own, and is folded.  Kernels of a
+    // pass list, us, all folded / none into real ops / by this rule: Fourier transform of 25 qubits
+    // complex64 1317 / 1111 / 1120, of 22 complex128 2506 / 1645 / 1700; Hadamards with 1.5 phases each
+    // between random qubits, 25 qubits complex64 2051 / 1718 / 1734; layers of RY and neighbouring CP,
+    // 25 qubits complex64 4088 / 6718 / 4088, 22 complex128 14382 / 20298 / 14379.
+    // Lists for one CTA (small states, the server) have no real path: there all is folded (10 layers of
+    // RY and CP on 10 qubits: 59 ops, 137 with the phases left).
+    std::vector<std::vector<int>> phases(relabel ? n : 0);   // per qubit, in each gap between its ops
+    auto gap = [&](int q, size_t i) { return (size_t)(std::upper_bound(on[q].begin(), on[q].end(), (int)i) - on[q].begin()); };
+    auto is_phase = [](const FOp& D) { return D.type == F_D && D.b >= 0 && !is_real(D); };
+    if (relabel) {
+      for (int q = 0; q < n; ++q) phases[q].assign(on[q].size() + 1, 0);
+      for (size_t i = 0; i < out.size(); ++i)
+        if (is_phase(out[i]))
+          for (int q : {out[i].a, out[i].b}) ++phases[q][gap(q, i)];
+    }
+    auto stays_real = [&](const FOp& D, size_t i, const FOp& G) {
+      return relabel && (G.type == F_G1 || G.type == F_G1C) && (G.t == D.a || G.t == D.b) && is_phase(D) &&
+             is_real(G) && phases[G.t][gap(G.t, i)] >= 2;
+    };
     for (size_t i = 0; i < out.size(); ++i) {
       if (out[i].type != F_D) continue;
       const FOp D = out[i];
@@ -285,8 +303,9 @@ void build_fused_ops(const qs_gate* gates, size_t ngates, int n, std::vector<FOp
         auto jt = std::lower_bound(L.begin(), L.end(), (int)i);
         if (jt != L.begin() && *(jt - 1) > before) before = *(jt - 1);
       }
-      bool done = after >= 0 && fold_into(D, out[(size_t)after], /*after=*/false);
-      if (!done && before >= 0) done = fold_into(D, out[(size_t)before], /*after=*/true);
+      bool done = after >= 0 && !stays_real(D, i, out[(size_t)after]) && fold_into(D, out[(size_t)after], /*after=*/false);
+      if (!done && before >= 0 && !stays_real(D, i, out[(size_t)before]))
+        done = fold_into(D, out[(size_t)before], /*after=*/true);
       if (done) dead[i] = 1;
     }
     size_t w = 0;
