@@ -229,9 +229,9 @@ __device__ __forceinline__ int src_bit(uint8_t src, uint8_t bit, uint64_t tile, 
 template <typename R, bool G2, bool REAL = true>
 __device__ __forceinline__ void apply_tile_op(C2<R>* v, const TileOp<R>* __restrict__ opp,
                                               uint64_t tile, int lane, int warp) {
-  // (the first 16 bytes with one load: kind, slot, csrc, cbit | dsrc, dbit, term | pad[0..3] | pad[4..7])
-  const uint4 hdr = *reinterpret_cast<const uint4*>(opp);
-  const uint32_t kind = hdr.x & 0xffu, slot = (hdr.x >> 8) & 0xffu, csrc = (hdr.x >> 16) & 0xffu, cbit = hdr.x >> 24;
+  uint4 hdr = {};   // kind, slot, csrc, cbit | dsrc, dbit, term | pad[0..3] | pad[4..7]
+  if (REAL) hdr = *reinterpret_cast<const uint4*>(opp);
+  const uint8_t kind = opp->kind, slot = opp->slot, csrc = opp->csrc, cbit = opp->cbit;
   if constexpr (G2) {
     if (kind == TK_G2) {   // reads its continuation opp[1]
       apply_g2(v, opp, lane);
@@ -396,7 +396,10 @@ __device__ __forceinline__ void apply_tile_op(C2<R>* v, const TileOp<R>* __restr
 // (ops with one bit in a register).  An op with both bits in registers
 // multiplies v directly.  flush() multiplies the collected diagonal into v once
 // the run ends.  Per op this is 1-2 complex products per thread instead of 16.
-template <typename R>
+// FLAG: a run that set no register-slot factor is multiplied by its scalar alone.  That saves FP64
+// instructions and runs beside TK_RUN; in the lean FP32 code it cost registers for nothing (25 qubits, 20
+// layers of Haar + CZ on tiles: 5.08 ms with it, 4.09 without).
+template <typename R, bool FLAG>
 struct DiagRun {
   C2<R> s, f0[2], f1[2], f2[2], f3[2];   // compile-time indices only (registers)
   bool slots;                            // a factor of a register slot was set (the same for the warp)
@@ -482,7 +485,7 @@ struct DiagRun {
   }
   template <bool TWO = false>
   __device__ __forceinline__ void flush(C2<R>* v, C2<R>* v2 = nullptr) {
-    if (!slots) {
+    if (FLAG && !slots) {
 #pragma unroll
       for (int r = 0; r < 16; ++r) {
         v[r] = cmul(v[r], s);
@@ -620,11 +623,11 @@ __device__ __forceinline__ void apply_cp_run(C2<R>* v, const TileOp<R>* __restri
 }
 
 // G2: the pass holds dense two-qubit ops; RUNS: it holds packed diagonal runs
-// (TK_RUN).  Each combination is its own instantiation, so that a pass without
-// them keeps the leaner code and register allocation.
+// (TK_RUN); REAL: its real ops take their own path.  Each combination is its own
+// instantiation, so that a pass without them keeps the leaner code and register allocation.
 // FP32: three CTAs on an SM, 80 registers each (with two, 7 % slower); only the leanest has to be told.
-template <typename R, bool G2, bool RUNS>
-__global__ void __launch_bounds__(kTileThreads, sizeof(R) == 4 && !G2 && !RUNS ? 3 : 0)
+template <typename R, bool G2, bool RUNS, bool REAL>
+__global__ void __launch_bounds__(kTileThreads, sizeof(R) == 4 && !G2 && !RUNS && REAL ? 3 : 0)
     tile_pass_kernel(C2<R>* __restrict__ psi, const __grid_constant__ TileParams<R> P) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C2<R>* sm = reinterpret_cast<C2<R>*>(smem_raw);
@@ -738,11 +741,11 @@ __global__ void __launch_bounds__(kTileThreads, sizeof(R) == 4 && !G2 && !RUNS ?
         continue;
       }
       if (k0 != TK_DIAG && k0 != TK_CP) {
-        apply_tile_op<R, G2>(v, ops + o, tile, lane, warp);
+        apply_tile_op<R, G2, REAL>(v, ops + o, tile, lane, warp);
         o += (G2 && k0 == TK_G2) ? 2 : 1;   // a dense two-qubit op spans two entries
         continue;
       }
-      DiagRun<R> dr;   // live only over the run
+      DiagRun<R, sizeof(R) == 8 || RUNS> dr;   // live only over the run
       dr.reset();
       uint4 hdr = *reinterpret_cast<const uint4*>(ops + o);
       do {
@@ -1039,7 +1042,7 @@ __global__ void __launch_bounds__(kTileThreads, sizeof(R) == 4 ? 2 : 1)
         o += (G2 && op->kind == TK_G2) ? 2 : 1;   // a dense two-qubit op spans two entries
         continue;
       }
-      DiagRun<R> dr;   // a run of diagonal U^dagger ops, on both states
+      DiagRun<R, true> dr;   // a run of diagonal U^dagger ops, on both states
       dr.reset();
       do {
         dr.template add<true>(vp, ops + o, tile, lane, warp, vl);
@@ -1856,10 +1859,17 @@ static bool pass_has_g2(const TileParams<R>& P) {
 
 // which op kinds a forward pass holds, walking op headers only (a dense
 // two-qubit op spans two slots; a TK_RUN header is followed by its entry slots,
-// whose bytes are not op headers)
+// whose bytes are not op headers).  real: whether the code with a path of its own for real
+// ops is the faster one.  FP64: always.  FP32: that code holds every complex op up by about a
+// tenth, so real ops have to be the most.  25 qubits, kernels of a circuit, us, without / with it: Haar
+// gates and CNOTs in equal numbers 6143 / 6866, RX and CNOT 3597 / 3959, Haar and CZ 4085 / 4083 (no
+// real op), Hadamards and CNOTs 3649 / 2884, Fourier transform 1196 / 1120.  Beside dense
+// two-qubit ops, whose code is large anyway, it wins from the first real op (300 mixed gates 2447 / 2346; SU(4)
+// brickwork, none real, 2753 / 2787).
 template <typename R>
-static void pass_kinds(const TileParams<R>& P, bool* g2, bool* runs) {
+static void pass_kinds(const TileParams<R>& P, bool* g2, bool* runs, bool* real) {
   *g2 = *runs = false;
+  int n_real = 0, n_complex = 0;
   const int nops = P.pass.n_stages > 0 ? P.stages[P.pass.n_stages - 1].op_end : 0;
   for (int o = 0; o < nops;) {
     const uint8_t k = P.ops[o].kind;
@@ -1870,33 +1880,41 @@ static void pass_kinds(const TileParams<R>& P, bool* g2, bool* runs) {
       *g2 = true;
       o += 2;
     } else {
+      if (k == TK_REG || k == TK_LANE) ++(P.ops[o].pad[2] ? n_real : n_complex);
       ++o;
     }
   }
+  *real = *g2 || n_real > n_complex;
 }
 
-template <typename R, bool G2, bool RUNS>
+template <typename R, bool G2, bool RUNS, bool REAL>
 static qs_status tile_launch_t(State* st, const TileParams<R>& P) {
   const uint64_t tiles = 1ull << (st->n - kTileBits);
   const size_t smem = sizeof(C2<R>) << kTileBits;
-  qs_status s = set_smem(tile_pass_kernel<R, G2, RUNS>, smem);
+  qs_status s = set_smem(tile_pass_kernel<R, G2, RUNS, REAL>, smem);
   if (s != QS_OK) return s;
-  tile_pass_kernel<R, G2, RUNS><<<(unsigned)tiles, kTileThreads, smem, st->stream>>>((C2<R>*)st->data, P);
+  tile_pass_kernel<R, G2, RUNS, REAL><<<(unsigned)tiles, kTileThreads, smem, st->stream>>>((C2<R>*)st->data, P);
   QS_CUDA(cudaGetLastError());
   return QS_OK;
 }
 
-template <typename R>
-static qs_status tile_launch_any(State* st, const TileParams<R>& P) {
-  bool g2 = false, runs = false;
-  pass_kinds(P, &g2, &runs);
-  if (g2) return runs ? tile_launch_t<R, true, true>(st, P) : tile_launch_t<R, true, false>(st, P);
-  return runs ? tile_launch_t<R, false, true>(st, P) : tile_launch_t<R, false, false>(st, P);
+template <typename R, bool REAL>
+static qs_status tile_launch_any(State* st, const TileParams<R>& P, bool g2, bool runs) {
+  if constexpr (REAL)   // (a pass with dense two-qubit ops always takes it)
+    if (g2) return runs ? tile_launch_t<R, true, true, REAL>(st, P) : tile_launch_t<R, true, false, REAL>(st, P);
+  return runs ? tile_launch_t<R, false, true, REAL>(st, P) : tile_launch_t<R, false, false, REAL>(st, P);
 }
 
 qs_status launch_tile_pass(State* st, const void* params) {
-  if (st->prec == QS_C64) return tile_launch_any(st, *(const TileParams<float>*)params);
-  return tile_launch_any(st, *(const TileParams<double>*)params);
+  bool g2 = false, runs = false, real = false;
+  if (st->prec == QS_C64) {
+    const TileParams<float>& P = *(const TileParams<float>*)params;
+    pass_kinds(P, &g2, &runs, &real);
+    return real ? tile_launch_any<float, true>(st, P, g2, runs) : tile_launch_any<float, false>(st, P, g2, runs);
+  }
+  const TileParams<double>& P = *(const TileParams<double>*)params;
+  pass_kinds(P, &g2, &runs, &real);
+  return tile_launch_any<double, true>(st, P, g2, runs);
 }
 
 template <typename R, bool G2>
