@@ -1211,14 +1211,19 @@ qs_status run_auto(State* st, const qs_gate* gates, size_t ngates, qs_stats* sta
     plan_chains(gates, ngates, st->n, plan, /*products=*/false);
     if (chains_dense(gates, plan)) return run_chains(st, gates, plan, stats, tm);
   }
+  // Density from the gates' patterns, and products only for the blocks that need them: the plan of
+  // chains above then costs less than it saves where it is given up (300 mixed gates on 20 qubits: 0.34 ms
+  // for it, and 0.44 in place of 1.25 ms here).
   std::vector<Block> blocks;
-  plan_blocks(gates, ngates, st->n, blocks);
+  plan_blocks(gates, ngates, st->n, blocks, /*products=*/false);
+  std::vector<char> is_dense(blocks.size());
+  for (size_t k = 0; k < blocks.size(); ++k) is_dense[k] = block_dense(gates, blocks[k]);
   // one or two dense blocks among sparse ones (the QFT's Hadamards among its
   // phases) may run on tile passes alone (auto_plan.h)
   {
     std::vector<FOp> fops;
     std::vector<int> vmap;
-    if (auto_all_tiles(gates, ngates, st->n, blocks, &fops, &vmap)) {
+    if (auto_all_tiles(gates, ngates, st->n, blocks, is_dense, &fops, &vmap)) {
       qs_stats part;
       std::memset(&part, 0, sizeof(part));
       qs_status s = run_tiled<float>(st, fops, vmap, &part, tm);
@@ -1235,8 +1240,6 @@ qs_status run_auto(State* st, const qs_gate* gates, size_t ngates, qs_stats* sta
       return s;
     }
   }
-  std::vector<char> is_dense(blocks.size());
-  for (size_t k = 0; k < blocks.size(); ++k) is_dense[k] = block_nonzeros(blocks[k]) > 512;
   if (chains) auto_short_runs(is_dense);
   size_t i = 0;
   qs_status s = QS_OK;
@@ -1253,6 +1256,7 @@ qs_status run_auto(State* st, const qs_gate* gates, size_t ngates, qs_stats* sta
     } else if (dense) {
       std::vector<Block> seg(std::make_move_iterator(blocks.begin() + (long)i),
                              std::make_move_iterator(blocks.begin() + (long)j));
+      parallel_for(seg.size(), 8, [&](size_t k) { block_product(gates, seg[k]); });
       s = run_block_list(st, seg, 1, stats, tm);
     } else {
       std::vector<qs_gate> seg;

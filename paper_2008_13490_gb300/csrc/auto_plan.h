@@ -15,6 +15,9 @@ namespace qs {
 // and *vmap (for the tiled run); false otherwise (the segment plan stands).
 bool auto_all_tiles(const qs_gate* gates, size_t ngates, int n, const std::vector<Block>& blocks,
                     std::vector<FOp>* fops, std::vector<int>* vmap);
+// the same for blocks whose density is known (their products are not needed)
+bool auto_all_tiles(const qs_gate* gates, size_t ngates, int n, const std::vector<Block>& blocks,
+                    const std::vector<char>& is_dense, std::vector<FOp>* fops, std::vector<int>* vmap);
 
 // A run of at most 4 sparse blocks beside dense ones costs a chain pass or two and a tile
 // pass as much or more, so in a circuit of mostly dense blocks (more than 3 for each block of

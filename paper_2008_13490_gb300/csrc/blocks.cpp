@@ -236,8 +236,15 @@ void plan_blocks(const qs_gate* gates, size_t ngates, int n, std::vector<Block>&
 
 bool auto_all_tiles(const qs_gate* gates, size_t ngates, int n, const std::vector<Block>& blocks,
                     std::vector<FOp>* fops, std::vector<int>* vmap) {
+  std::vector<char> is_dense(blocks.size());
+  for (size_t i = 0; i < blocks.size(); ++i) is_dense[i] = block_nonzeros(blocks[i]) > 512;
+  return auto_all_tiles(gates, ngates, n, blocks, is_dense, fops, vmap);
+}
+
+bool auto_all_tiles(const qs_gate* gates, size_t ngates, int n, const std::vector<Block>& blocks,
+                    const std::vector<char>& is_dense, std::vector<FOp>* fops, std::vector<int>* vmap) {
   int dense = 0;
-  for (const Block& b : blocks) dense += block_nonzeros(b) > 512 ? 1 : 0;
+  for (char d : is_dense) dense += d;
   if (dense < 1 || dense > 2 || dense == (int)blocks.size()) return false;
   // tile passes and remaps of a gate list, fused as the default method fuses it
   auto count = [&](const std::vector<qs_gate>& seg, int* passes, int* remaps) {
@@ -251,7 +258,7 @@ bool auto_all_tiles(const qs_gate* gates, size_t ngates, int n, const std::vecto
   for (size_t i = 0; i < blocks.size();) {   // the runs of sparse blocks
     std::vector<qs_gate> seg;
     size_t j = i;
-    while (j < blocks.size() && block_nonzeros(blocks[j]) <= 512) {
+    while (j < blocks.size() && !is_dense[j]) {
       for (size_t gi : blocks[j].gate_idx) seg.push_back(gates[gi]);
       ++j;
     }
