@@ -110,7 +110,7 @@ __device__ __forceinline__ uint64_t digits_of(uint32_t lo, uint32_t hi, uint32_t
   const uint32_t e = (hi >> 20) & 0x7ffu;
   uint32_t s = E - e;
   uint64_t m = ((uint64_t)((hi & 0xfffffu) | 0x100000u) << 32 | lo) << 2;
-  m = s < 64u ? m >> s : 0ull;   // (x = 0 has e = 0, and E >= kMinExp)
+  m = s < 64u ? m >> s : 0ull;   // (x = 0 has e = 0, and E >= kF64MinExp)
   const uint64_t sign = (uint64_t)(int64_t)((int32_t)hi >> 31);
   // bias: 256 in each of the five 9-bit digits, 512 in the top one; plus 1/2 for the rounding
   constexpr uint64_t kBias = 256ull * (1ull + (1ull << 9) + (1ull << 18) + (1ull << 27) + (1ull << 36)) + (512ull << 45);
@@ -128,7 +128,6 @@ __device__ __forceinline__ uint32_t digit_pair(uint64_t a, uint64_t b) {
   asm("add.rn.f16x2 %0, %1, %2;" : "=r"(r) : "r"(u), "r"(I == 0 ? 0xe600e600u : 0xe500e500u));
   return r;
 }
-constexpr uint32_t kMinExp = 128, kMaxExp = 1950;   // rows below are zero, above (and NaN) not a number
 
 __global__ void __launch_bounds__(kThreads, 1)
     block_f64_kernel(const __grid_constant__ F64Pass P, const __grid_constant__ CUtensorMap tmap,
@@ -207,7 +206,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (!ok) break;
       top = max(max(s_max[0][m], s_max[1][m]), max(s_max[2][m], s_max[3][m]));
       uint32_t E = top >> 20;
-      const bool bad = E > kMaxExp, zero = E < kMinExp;
+      const bool bad = E > kF64MaxExp, zero = E < kF64MinExp;
       if (bad || zero) E = 2047u + 64u;   // every digit zero: the shift is 64 or more
 #pragma unroll
       for (int part = 0; part < 2; ++part) {   // real parts, then imaginary

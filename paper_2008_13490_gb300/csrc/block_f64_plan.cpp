@@ -185,7 +185,7 @@ bool f64_b_operand(const qs_gate* gates, const Block& b, unsigned char* out, int
       if (!std::isfinite(U.rh[r][c]) || !std::isfinite(U.ih[r][c])) return false;
       big = std::max(big, std::max(std::abs(U.rh[r][c]), std::abs(U.ih[r][c])));
     }
-  if (!(big > 1e-30 && big < 1e30)) return false;
+  if (!(big > std::ldexp(1.0, -kF64MaxEntryExp) && big < std::ldexp(1.0, kF64MaxEntryExp))) return false;
   int e = 0;
   const double f = std::frexp(big, &e);   // big = f 2^e, 1/2 <= f < 1
   *vs = 55 - (f == 0.5 ? e - 1 : e);
