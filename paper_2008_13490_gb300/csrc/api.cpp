@@ -1153,14 +1153,15 @@ qs_status run_f64_blocks(State* st, const qs_gate* gates, size_t ngates, qs_stat
   std::vector<F64Pass> passes(blocks.size());
   for (size_t i = 0; i < blocks.size(); ++i)
     if (!f64_pass_desc(st->n, blocks[i].q, passes[i])) return QS_EUNSUPPORTED;
-  const size_t bytes = 16 + blocks.size() * (size_t)kF64B;   // status word, B operands
+  const size_t bytes = 16 + blocks.size() * (size_t)kF64Op;   // status word, operands
   unsigned char* host = nullptr;
   qs_status s = upload_begin(st, bytes, &host);
   if (s != QS_OK) return s;
   std::memset(host, 0, 16);
   std::vector<char> fits(blocks.size());
   parallel_for(blocks.size(), 2, [&](size_t i) {
-    fits[i] = f64_b_operand(gates, blocks[i], host + 16 + i * kF64B, &passes[i].vs);
+    unsigned char* const at = host + 16 + i * kF64Op;
+    fits[i] = f64_b_operand(gates, blocks[i], at, &passes[i].vs, (cd*)(at + kF64B));
   });
   if (std::find(fits.begin(), fits.end(), (char)0) != fits.end()) return QS_EUNSUPPORTED;
   s = launch_f64_setup();
@@ -1169,7 +1170,7 @@ qs_status run_f64_blocks(State* st, const qs_gate* gates, size_t ngates, qs_stat
   s = upload_part(st, 0, bytes, true);
   for (size_t i = 0; i < blocks.size() && s == QS_OK; ++i) {
     tm.before(4);
-    s = launch_f64_pass(st, passes[i], dev + 16 + i * kF64B, (int*)dev);
+    s = launch_f64_pass(st, passes[i], dev + 16 + i * kF64Op, (int*)dev);
     tm.after();
   }
   if (s != QS_OK) {

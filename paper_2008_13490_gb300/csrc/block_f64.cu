@@ -1,17 +1,20 @@
 // Dense 5-qubit blocks of complex128 states on the tcgen05 tensor cores.
 //
-// FP64 runs at 1/64 of the FP32 rate on this GPU (1.06 TFLOP/s), so a complex128 circuit on
+// FP64 runs at 1/75 of the FP32 rate on this GPU (1.06 TFLOP/s), so a complex128 circuit on
 // tile passes is bound by it: 278 ms for 40 Haar + CZ layers at 25 qubits, 0.5 % of HBM.  Here
 // the product y = U x of a row of 32 amplitudes is formed in integers instead, exactly but
-// for one rounding of the inputs and one of the result:
+// for one rounding of the inputs and one of the result (the error-free splitting of matrix products of
+// Ozaki, Ogita, Oishi and Rump, Numer. Algorithms 59 (2012), with digits on a common exponent):
 //   - the 64 real parts of a row become 54-bit integers on the exponent of the row's largest
 //     (rounded to nearest; the row's own scale), in six balanced digits: a top one of |d| <= 512
 //     and five of 9 bits, |d| <= 256; the block's entries likewise (55 bits, block_f64_plan.cpp);
 //   - digits are FP16 integers, so a tcgen05.mma of one digit slice by another sums up to 64
 //     products of at most 2^19 in FP32 exactly; slices (i, j) of the same order s = i + j share an
 //     accumulator, seven orders s = 0..6 (26 slice products) reach 2^-60 of the row;
-//   - the epilogue adds the orders as 64-bit integers and converts once to FP64.
-// 25 qubits, 40 layers: 32 ms (81 blocks, 0.35 ms each) against 278 ms.  Error against 112-bit
+//   - the epilogue adds the orders as 64-bit integers and converts once to FP64;
+//   - rows whose amplitudes do not share an exponent well, or leave its range, are multiplied in FP64
+//     arithmetic instead (row_in_fp64; the bounds are in block_f64.h).
+// 25 qubits, 40 layers: 33 ms (81 blocks, 0.37 ms each) against 278 ms.  Error against 112-bit
 // arithmetic at 15 qubits, 80 layers: 8.9e-16, against 2.7e-15 of FP64 arithmetic gate by gate.
 //
 // A persistent CTA (one per SM) takes a tile of 2^12 amplitudes (128 rows) at a time:
@@ -129,14 +132,61 @@ __device__ __forceinline__ uint32_t digit_pair(uint64_t a, uint64_t b) {
   return r;
 }
 
+// A row multiplied in FP64 arithmetic, where `mine`: the eight outputs from u on (rows of 32 entries) of
+// the row at `row` in shared memory, to columns `first` and on.  Entries that are zero are left out, so that an
+// infinity or a NaN goes only where gates take it.  All 128 threads of the row's warps call this.  (Rolled
+// loops and a local array: the code around it has no registers to spare.)
+__device__ __forceinline__ void row_in_fp64(bool mine, const double2* __restrict__ u, uint32_t row, uint32_t first,
+                                            const F64Pass& P, int barrier) {
+  double2 y[8];
+  if (mine) {
+#pragma unroll 1
+    for (int r = 0; r < 8; ++r) {
+      double re = 0.0, im = 0.0;
+      uint32_t e = row;
+#pragma unroll 1
+      for (int k = 0, c = 0; k < 32; ++k) {   // columns in Gray-code order
+        if (k) {
+          const int j = __ffs(k) - 1;
+          e ^= 16u * P.col[j];
+          c ^= 1 << j;
+        }
+        const uint4 v = lds128(e);
+        const double xr = __hiloint2double((int)v.y, (int)v.x), xi = __hiloint2double((int)v.w, (int)v.z);
+        const double2 m = u[32 * r + c];
+        if (m.x != 0.0) {
+          re = fma(m.x, xr, re);
+          im = fma(m.x, xi, im);
+        }
+        if (m.y != 0.0) {
+          re = fma(-m.y, xi, re);
+          im = fma(m.y, xr, im);
+        }
+      }
+      y[r] = make_double2(re, im);
+    }
+  }
+  __syncwarp();
+  bar_sync(barrier, 128);
+#pragma unroll 1
+  for (int r = 0; mine && r < 8; ++r) {
+    const uint32_t e = row ^ first ^ 16u * ((r & 1 ? P.col[0] : 0u) ^ (r & 2 ? P.col[1] : 0u) ^ (r & 4 ? P.col[2] : 0u));
+    const double2 v = y[r];
+    sts128(e, make_uint4((uint32_t)__double2loint(v.x), (uint32_t)__double2hiint(v.x), (uint32_t)__double2loint(v.y),
+                         (uint32_t)__double2hiint(v.y)));
+  }
+  __syncwarp();
+}
+
 __global__ void __launch_bounds__(kThreads, 1)
     block_f64_kernel(const __grid_constant__ F64Pass P, const __grid_constant__ CUtensorMap tmap,
                      const unsigned char* __restrict__ bmat, uint32_t ntiles, int* __restrict__ status) {
+  const double2* __restrict__ umat = reinterpret_cast<const double2*>(bmat + kF64B);   // the block in FP64
   extern __shared__ __align__(128) unsigned char smem_raw[];
   __shared__ __align__(8) uint64_t full[2], done[2], afull, dfull[2], dempty[2], drain;
   __shared__ uint32_t tmem_slot;
   __shared__ int s_fail;
-  __shared__ uint32_t s_max[4][128];
+  __shared__ uint32_t s_exp[4][128];   // by quarter and row: exponents of the largest and smallest amplitude
   const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
   const uint32_t bsm = smem_u32(smem_raw);
   const uint32_t slots = (bsm + (uint32_t)kF64B + (kSlotBytes - 1u)) & ~(kSlotBytes - 1u);
@@ -190,7 +240,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       const uint32_t slot = i & 1u, sbase = slots + slot * (uint32_t)kSlotBytes;
       bool ok = alive && warp_wait(&full[slot], (i >> 1) & 1u, &s_fail);
       uint4 x[8];
-      uint32_t top = 0;
+      uint32_t top = 0, low = 0xffffffffu;
       if (ok) {
         uint32_t e = sbase + 16u * (rbase ^ cq);
 #pragma unroll
@@ -199,15 +249,21 @@ __global__ void __launch_bounds__(kThreads, 1)
           x[k ^ (k >> 1)] = lds128(e);
         }
 #pragma unroll
-        for (int k = 0; k < 8; ++k) top = max(top, max(x[k].y & 0x7fffffffu, x[k].w & 0x7fffffffu));
-        s_max[quarter][m] = top;
+        for (int k = 0; k < 8; ++k) {
+          const uint32_t a = max(x[k].y & 0x7fffffffu, x[k].w & 0x7fffffffu);
+          top = max(top, a);
+          low = min(low, a - 1u);   // (zero, and what is below 2^-1042: the largest)
+        }
+        s_exp[quarter][m] = (top >> 20) << 16 | (0xfffu - (low >> 20));
       }
       ok = !bar_or(1, kWorkers, !ok);
       if (!ok) break;
-      top = max(max(s_max[0][m], s_max[1][m]), max(s_max[2][m], s_max[3][m]));
-      uint32_t E = top >> 20;
-      const bool bad = E > kF64MaxExp, zero = E < kF64MinExp;
-      if (bad || zero) E = 2047u + 64u;   // every digit zero: the shift is 64 or more
+      const uint32_t ex = __vmaxu2(__vmaxu2(s_exp[0][m], s_exp[1][m]), __vmaxu2(s_exp[2][m], s_exp[3][m]));
+      const uint32_t least = 0xfffu - (ex & 0xffffu);   // 0xfff: a row of zeros
+      uint32_t E = ex >> 16;
+      // rows that the integers do not hold (kF64Spread)
+      const bool apart = least != 0xfffu && (E > kF64MaxExp || E < kF64MinExp || E - least > kF64Spread);
+      if (apart || least == 0xfffu) E = 2047u + 64u;   // every digit zero: the shift is 64 or more
 #pragma unroll
       for (int part = 0; part < 2; ++part) {   // real parts, then imaginary
         uint32_t w[kF64Slices][4];
@@ -228,6 +284,10 @@ __global__ void __launch_bounds__(kThreads, 1)
           tmem_st4(lanes + kColA + 32u * s + 8u * (uint32_t)quarter + 4u * part, w[s]);
       }
       tmem_wait_st();
+      // Rows apart are read whole before any of the row's four threads writes to it (their warps, w and
+      // w + 4 .., agree on whether there are any), and all rows are written after this arrival.
+      if (__any_sync(0xffffffffu, apart))
+        row_in_fp64(apart, umat + 256 * quarter, sbase + 16u * rbase, 16u * cq, P, 2 + (warp & 3));
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       mbar_arrive(&afull);
       // the outputs, a quarter (8 amplitudes a row) at a time: this thread's are 8 q + 2 quarter
@@ -262,15 +322,16 @@ __global__ void __launch_bounds__(kThreads, 1)
           const double d = __ll2double_rn(y);
           uint32_t hi = (uint32_t)__double2hiint(d), lo = (uint32_t)__double2loint(d);
           if (hi | lo) hi += exp_add;
-          if (bad) hi = 0x7ff80000u;
           out[2 * k] = lo;
           out[2 * k + 1] = hi;
         }
         // (in place: every row has been read when the first accumulators are full)
         uint32_t c = (q & 1u ? cb[3] : 0u) ^ (q & 2u ? cb[4] : 0u) ^ (quarter & 1 ? cb[1] : 0u) ^ (quarter & 2 ? cb[2] : 0u);
         const uint32_t e = (sbase + 16u * rbase) ^ c;
-        sts128(e, make_uint4(out[0], out[1], out[2], out[3]));
-        sts128(e ^ cb[0], make_uint4(out[4], out[5], out[6], out[7]));
+        if (!apart) {
+          sts128(e, make_uint4(out[0], out[1], out[2], out[3]));
+          sts128(e ^ cb[0], make_uint4(out[4], out[5], out[6], out[7]));
+        }
       }
       alive = ok;
       if (!ok) continue;

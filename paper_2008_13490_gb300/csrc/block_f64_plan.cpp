@@ -176,9 +176,11 @@ void pair_product(const qs_gate* gates, const Block& b, PairMatrix& U) {
 // bottom and a top one (|d| <= 1024), FP16 integers.  Row n = 16 q + 2 r + part is the real
 // (part 0) or imaginary part of output 8 q + r; K = 16 j + k: the real parts of columns
 // 8 j .. 8 j + 7, then the imaginary ones.  K-major core matrices, no swizzle.
-bool f64_b_operand(const qs_gate* gates, const Block& b, unsigned char* out, int32_t* vs) {
+bool f64_b_operand(const qs_gate* gates, const Block& b, unsigned char* out, int32_t* vs, cd* matrix) {
   PairMatrix U;
   pair_product(gates, b, U);
+  for (int k = 0; matrix && k < 32 * 32; ++k)
+    matrix[k] = cd(U.rh[k >> 5][k & 31] + U.rl[k >> 5][k & 31], U.ih[k >> 5][k & 31] + U.il[k >> 5][k & 31]);
   double big = 0;
   for (int r = 0; r < 32; ++r)
     for (int c = 0; c < 32; ++c) {

@@ -218,9 +218,6 @@ __device__ __forceinline__ void box_store4(const CUtensorMap* map, int c0, int c
       "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(smem_u32(src))
       : "memory");
 }
-__device__ __forceinline__ void bar_sync(int id, int nthreads) {
-  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
-}
 // BOX: the pass writes its output back with tensor stores (BlockPass flag bit 1);
 // a separate instantiation, so that each variant keeps its own register budget
 template <int MODE, bool BOX>

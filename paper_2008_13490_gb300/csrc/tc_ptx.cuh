@@ -109,6 +109,9 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* b, uint32_t parity, const in
   }
   return false;
 }
+__device__ __forceinline__ void bar_sync(int id, int nthreads) {
+  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
+}
 // OR of a predicate over the threads of a named barrier (all of them arrive)
 __device__ __forceinline__ bool bar_or(int id, int nthreads, bool v) {
   uint32_t r;

@@ -9,6 +9,7 @@ import pytest
 
 import workloads as W
 from conftest import ROOT
+from oracle import statevector as SV
 
 
 def _dense(qubits, layers, g):
@@ -20,20 +21,24 @@ def _dense(qubits, layers, g):
     return ops
 
 
-@pytest.fixture(scope="module")
-def scale_exe(tmp_path_factory):
+def _compile(tmp_path_factory, name):
     if shutil.which("g++") is None:
         pytest.skip("g++ not available")
     from paper_2008_13490_gb300 import _build
     lib = _build.build()
     libdir = os.path.dirname(lib)
-    exe = tmp_path_factory.mktemp("f64s") / "f64_scale_check"
+    exe = tmp_path_factory.mktemp("f64") / name
     cuda_inc = os.path.join(os.environ.get("CUDA_HOME", "/usr/local/cuda"), "include")
-    subprocess.run(["g++", "-O2", "-std=c++17", os.path.join(ROOT, "tests", "f64_scale_check.cpp"),
+    subprocess.run(["g++", "-O2", "-std=c++17", os.path.join(ROOT, "tests", name + ".cpp"),
                     "-I", os.path.join(ROOT, "paper_2008_13490_gb300", "csrc"), "-I", os.path.join(ROOT, "include"),
                     "-I", cuda_inc, "-o", str(exe), "-L", libdir, "-lqsim", f"-Wl,-rpath,{libdir}"],
                    check=True, capture_output=True, text=True)
     return exe
+
+
+@pytest.fixture(scope="module")
+def scale_exe(tmp_path_factory):
+    return _compile(tmp_path_factory, "f64_scale_check")
 
 
 def test_exponent_fields_of_accepted_blocks(scale_exe):
@@ -69,3 +74,84 @@ def test_matrices_far_from_unitary(qs, size, amp):
         assert stats["tile_launches"] > 0
     assert np.array_equal(outs[0].view(np.uint64), outs[1].view(np.uint64)) or \
         np.array_equal(outs[0], outs[1], equal_nan=True)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("qubits", [[9, 10, 11, 12, 13], [0, 1, 2, 3, 4], [1, 4, 6, 9, 13]])
+def test_rows_that_the_integers_do_not_hold(qs, qubits):
+    # one dense block; rows are the values of the other nine qubits.  Rows of zeros stay zero, a scaled row gives
+    # the scaled result, a row with one amplitude gives that column; rows apart (tiny, huge, subnormal, of a
+    # wide range, with an infinity or a NaN) give what FP64 gives, and only they
+    n, g = 14, W.rng(7)
+    ops = _dense(qubits, 6, g)
+    others = [q for q in range(n) if q not in qubits]
+    J = np.arange(1 << n)
+    row = sum(((J >> q) & 1) << k for k, q in enumerate(others))
+    col = sum(((J >> q) & 1) << k for k, q in enumerate(qubits))
+    at = np.zeros((512, 32), dtype=np.int64)
+    at[row, col] = J
+    x = W.random_state(n, g)[at] * 2.0 ** (n / 2)
+    x[3] = 0
+    x[4] = x[5] * 2.0 ** -200
+    x[6, 9] = np.nan
+    x[7, 20] = np.inf
+    x[8] = 0
+    x[8, 11] = 0.5
+    x[9] = x[5] * 2.0 ** -950          # below the integers' exponents
+    x[10] = x[5] * 2.0 ** 1000         # above them
+    x[11] = 0
+    x[11, 4] = 3e-310                  # subnormal
+    x[12:40] = x[5] * np.exp2(-np.arange(32))[g.permutation(32)] ** (np.arange(28)[:, None] / 4)   # ever wider
+    x[40, 1:] *= 1e-30
+    x[511, 31] = 1e-25
+    psi = np.empty(1 << n, dtype=np.complex128)
+    psi[at] = x
+    st = qs.State(n, qs.QS_C128)
+    qs.sv_copy_in(st, psi)
+    stats = qs.sv_apply_circuit(st, ops)
+    out = qs.sv_copy_out(st)[at]
+    st.close()
+    assert stats["passes"] == stats["ops_fused"] == 1 and stats["tile_launches"] == 0
+    assert stats["flops"] == 256.0 * 2 ** n
+    # the block, from the oracle's columns
+    U = np.stack([SV.apply_circuit(SV.basis(5, j) if j else SV.basis(5), 5,
+                                   [(k, tuple(qubits.index(q) for q in qq), p, m) for k, qq, p, m in ops])
+                  for j in range(32)], axis=1)
+    assert np.all(U != 0)
+    assert np.all(out[3] == 0)
+    assert np.array_equal(out[4], out[5] * 2.0 ** -200)
+    for r in (6, 7):
+        assert not np.isfinite(out[r]).any()
+    ok = np.array([r for r in range(512) if r not in (6, 7)])
+    assert np.isfinite(out[ok]).all()
+    # relative to the largest amplitude of the row: 32 products and sums of a few 2^-53 each (the oracle's U
+    # as many); subnormal results to their spacing
+    want = x[ok] @ U.T
+    big = np.abs(x[ok]).max(axis=1, keepdims=True)
+    assert np.all(np.abs(out[ok] - want) <= 64 * 2.0 ** -53 * big + 4 * 5e-324 * 32)
+
+
+@pytest.mark.gpu
+def test_small_amplitudes_beside_large_ones(qs):
+    # a state whose qubits 0..3 hardly leave zero, then dense blocks on others: each amplitude keeps its own
+    # digits (2^-34 of it in each block), also where a block takes idle qubits along
+    n, layers, g = 15, 8, W.rng(23)
+    t = 1e-4
+    small = np.array([1.0 + 0j])
+    for q in range(4):
+        small = np.kron(np.array([np.cos(t), -1j * np.sin(t)]), small)
+    rest = W.random_state(n - 4, g)
+    psi = np.kron(rest, small)
+    ops = []
+    for layer in range(layers):
+        ops += [("MAT1", (q,), (), W.haar_su2(g)) for q in range(4, n)]
+        ops += [("CZ", (q, q + 1), (), None) for q in range(4 + layer % 2, n - 1, 2)]
+    st = qs.State(n, qs.QS_C128)
+    qs.sv_copy_in(st, psi)
+    stats = qs.sv_apply_circuit(st, ops)
+    out = qs.sv_copy_out(st).reshape(-1, 16)
+    st.close()
+    assert stats["passes"] == stats["ops_fused"] and stats["tile_launches"] == 0
+    ref = SV.apply_circuit(rest.copy(), n - 4, [(k, tuple(q - 4 for q in qq), p, m) for k, qq, p, m in ops])
+    for j in range(16):
+        assert np.linalg.norm(out[:, j] / small[j] - ref) <= 4 * np.sqrt(stats["passes"]) * 2.0 ** -34, j
