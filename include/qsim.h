@@ -123,8 +123,13 @@ typedef enum {
    * only one or two dense blocks, the whole circuit runs on tile passes when that
    * takes no more tile passes and remaps than the sparse runs alone (the blocks'
    * sweeps are saved).  Larger complex128 states: circuits of mostly dense blocks run
-   * block by block on the tensor cores too, in exact integer slices of the FP64
-   * values (one rounding per block and amplitude).  Everything else uses
+   * block by block on the tensor cores too, in exact integer slices: the amplitudes that
+   * a block mixes are rounded to 2^-54 of their largest, the block's entries to 2^-55 of
+   * its largest, and the result once more, which is less than FP64 arithmetic rounds gate
+   * by gate.  An amplitude of 2^-k of the largest that it is mixed with keeps 54 - k
+   * bits of its own: where one is below 2^-20 of it FP64 arithmetic takes the place of the integers, and a
+   * block with an entry below 2^-20 of its largest runs on tile passes.  QS_METHOD_TILED
+   * keeps FP64's relative precision of every amplitude.  Everything else uses
    * QS_METHOD_TILED.
    * Synchronous like the block methods for complex64 states with n >= 12, and where
    * complex128 blocks run. */

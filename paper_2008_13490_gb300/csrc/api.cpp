@@ -1139,36 +1139,22 @@ qs_status run_blocks(State* st, const qs_gate* gates, size_t ngates, int mode, q
   return run_block_list(st, blocks, mode, stats, tm);
 }
 
-// QS_METHOD_AUTO, complex128, n > kSmallAutoBits: circuits of mostly dense blocks (at least three for each
-// sparse one) run block by block on the tensor cores (block_f64.cu).  QS_EUNSUPPORTED, with
-// nothing launched, for others and for matrices that the integer slices do not take: they run
-// on tile passes.
-qs_status run_f64_blocks(State* st, const qs_gate* gates, size_t ngates, qs_stats* stats, KernelTimer& tm) {
-  if (!chains_likely(gates, ngates)) return QS_EUNSUPPORTED;
-  std::vector<Block> blocks;
-  plan_blocks(gates, ngates, st->n, blocks, /*products=*/false);
-  size_t dense = 0;
-  for (const Block& b : blocks) dense += block_dense(gates, b);
-  if (dense == 0 || dense < 3 * (blocks.size() - dense)) return QS_EUNSUPPORTED;
-  std::vector<F64Pass> passes(blocks.size());
-  for (size_t i = 0; i < blocks.size(); ++i)
-    if (!f64_pass_desc(st->n, blocks[i].q, passes[i])) return QS_EUNSUPPORTED;
-  const size_t bytes = 16 + blocks.size() * (size_t)kF64Op;   // status word, operands
-  unsigned char* host = nullptr;
-  qs_status s = upload_begin(st, bytes, &host);
-  if (s != QS_OK) return s;
+// One sweep per block over blocks [0, count), their operands (kF64Op bytes each) at `ops`, or null: then
+// they stand in the pinned buffer already, from byte 16 on.
+qs_status run_f64_list(State* st, const F64Pass* passes, size_t count, const unsigned char* ops, qs_stats* stats,
+                       KernelTimer& tm) {
+  const size_t bytes = 16 + count * (size_t)kF64Op;   // status word, operands
+  unsigned char* host = (unsigned char*)st->hostbuf;
+  qs_status s = QS_OK;
+  if (ops) {
+    s = upload_begin(st, bytes, &host);
+    if (s != QS_OK) return s;
+    std::memcpy(host + 16, ops, bytes - 16);
+  }
   std::memset(host, 0, 16);
-  std::vector<char> fits(blocks.size());
-  parallel_for(blocks.size(), 2, [&](size_t i) {
-    unsigned char* const at = host + 16 + i * kF64Op;
-    fits[i] = f64_b_operand(gates, blocks[i], at, &passes[i].vs, (cd*)(at + kF64B));
-  });
-  if (std::find(fits.begin(), fits.end(), (char)0) != fits.end()) return QS_EUNSUPPORTED;
-  s = launch_f64_setup();
-  if (s != QS_OK) return s;
   unsigned char* dev = (unsigned char*)st->opbuf;
   s = upload_part(st, 0, bytes, true);
-  for (size_t i = 0; i < blocks.size() && s == QS_OK; ++i) {
+  for (size_t i = 0; i < count && s == QS_OK; ++i) {
     tm.before(4);
     s = launch_f64_pass(st, passes[i], dev + 16 + i * kF64Op, (int*)dev);
     tm.after();
@@ -1186,13 +1172,83 @@ qs_status run_f64_blocks(State* st, const qs_gate* gates, size_t ngates, qs_stat
     return status == QS_ETIMEOUT ? QS_ETIMEOUT : QS_ECUDA;
   }
   if (stats) {
-    stats->ops_fused += (int64_t)blocks.size();
-    stats->passes += (int64_t)blocks.size();
-    stats->launches += (int64_t)blocks.size();
-    stats->flops += 256.0 * std::ldexp(1.0, st->n) * (double)blocks.size();
+    stats->ops_fused += (int64_t)count;
+    stats->passes += (int64_t)count;
+    stats->launches += (int64_t)count;
+    stats->flops += 256.0 * std::ldexp(1.0, st->n) * (double)count;
     stats->upload_bytes += (int64_t)bytes;
   }
   return QS_OK;
+}
+
+// The gates of blocks [i, j) on tile passes, added to stats.
+template <typename R>
+qs_status run_tile_segment(State* st, const qs_gate* gates, const std::vector<Block>& blocks, size_t i, size_t j,
+                           qs_stats* stats, KernelTimer& tm) {
+  std::vector<qs_gate> seg;
+  for (size_t k = i; k < j; ++k)
+    for (size_t gi : blocks[k].gate_idx) seg.push_back(gates[gi]);
+  std::vector<FOp> fops;
+  std::vector<int> vmap;
+  build_fused_ops(seg.data(), seg.size(), st->n, fops, vmap, /*fuse=*/true, /*relabel=*/true);
+  qs_stats part;
+  std::memset(&part, 0, sizeof(part));
+  const qs_status s = run_tiled<R>(st, fops, vmap, &part, tm);
+  if (stats) {
+    stats->ops_fused += part.ops_fused;
+    stats->passes += part.passes;
+    stats->launches += part.launches;
+    stats->tile_launches += part.tile_launches;
+    stats->tile_flops += part.tile_flops;
+    stats->flops += part.flops;
+    stats->upload_bytes += part.upload_bytes;
+  }
+  return s;
+}
+
+// QS_METHOD_AUTO, complex128, n > kSmallAutoBits: circuits of mostly dense blocks (at least three for each
+// other one) run block by block on the tensor cores (block_f64.cu), and blocks whose matrices the
+// integer slices do not take (f64_b_operand) gate by gate on tile passes between them.
+// QS_EUNSUPPORTED, with nothing launched, for other circuits: they run on tile passes.
+qs_status run_f64_blocks(State* st, const qs_gate* gates, size_t ngates, qs_stats* stats, KernelTimer& tm) {
+  if (!chains_likely(gates, ngates)) return QS_EUNSUPPORTED;
+  std::vector<Block> blocks;
+  plan_blocks(gates, ngates, st->n, blocks, /*products=*/false);
+  const size_t nb = blocks.size();
+  std::vector<char> is_dense(nb), fits(nb);
+  auto mostly = [&](const std::vector<char>& also) {
+    size_t dense = 0;
+    for (size_t i = 0; i < nb; ++i) dense += is_dense[i] && also[i];
+    return dense > 0 && dense >= 3 * (nb - dense);
+  };
+  for (size_t i = 0; i < nb; ++i) is_dense[i] = block_dense(gates, blocks[i]);
+  if (!mostly(is_dense)) return QS_EUNSUPPORTED;
+  std::vector<F64Pass> passes(nb);
+  for (size_t i = 0; i < nb; ++i)
+    if (!f64_pass_desc(st->n, blocks[i].q, passes[i])) return QS_EUNSUPPORTED;
+  unsigned char* host = nullptr;
+  qs_status s = upload_begin(st, 16 + nb * (size_t)kF64Op, &host);
+  if (s != QS_OK) return s;
+  parallel_for(nb, 2, [&](size_t i) {
+    unsigned char* const at = host + 16 + i * kF64Op;
+    fits[i] = f64_b_operand(gates, blocks[i], at, &passes[i].vs, (cd*)(at + kF64B));
+  });
+  if (!mostly(fits)) return QS_EUNSUPPORTED;
+  s = launch_f64_setup();
+  if (s != QS_OK) return s;
+  if (std::find(fits.begin(), fits.end(), (char)0) == fits.end())
+    return run_f64_list(st, passes.data(), nb, nullptr, stats, tm);
+  // (the tile passes' uploads take the pinned buffer)
+  const std::vector<unsigned char> ops(host + 16, host + 16 + nb * (size_t)kF64Op);
+  for (size_t i = 0; i < nb && s == QS_OK;) {
+    size_t j = i;
+    while (j < nb && fits[j] == fits[i]) ++j;
+    s = fits[i] ? run_f64_list(st, passes.data() + i, j - i, ops.data() + i * kF64Op, stats, tm)
+                : run_tile_segment<double>(st, gates, blocks, i, j, stats, tm);
+    if (s == QS_EUNSUPPORTED) s = QS_ECUDA;   // (something has been launched)
+    i = j;
+  }
+  return s;
 }
 
 // QS_METHOD_AUTO (complex64, larger states than kSmallAutoBits allows): the circuit is cut into 5-qubit blocks;
@@ -1260,24 +1316,7 @@ qs_status run_auto(State* st, const qs_gate* gates, size_t ngates, qs_stats* sta
       parallel_for(seg.size(), 8, [&](size_t k) { block_product(gates, seg[k]); });
       s = run_block_list(st, seg, 1, stats, tm);
     } else {
-      std::vector<qs_gate> seg;
-      for (size_t k = i; k < j; ++k)
-        for (size_t gi : blocks[k].gate_idx) seg.push_back(gates[gi]);
-      std::vector<FOp> fops;
-      std::vector<int> vmap;
-      build_fused_ops(seg.data(), seg.size(), st->n, fops, vmap, /*fuse=*/true, /*relabel=*/true);
-      qs_stats part;
-      std::memset(&part, 0, sizeof(part));
-      s = run_tiled<float>(st, fops, vmap, &part, tm);
-      if (stats) {
-        stats->ops_fused += part.ops_fused;
-        stats->passes += part.passes;
-        stats->launches += part.launches;
-        stats->tile_launches += part.tile_launches;
-        stats->tile_flops += part.tile_flops;
-        stats->flops += part.flops;
-        stats->upload_bytes += part.upload_bytes;
-      }
+      s = run_tile_segment<float>(st, gates, blocks, i, j, stats, tm);
     }
     i = j;
   }

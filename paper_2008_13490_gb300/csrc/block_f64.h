@@ -24,6 +24,10 @@ constexpr uint32_t kF64MinExp = 128, kF64MaxExp = 1950;   // E
 // not come: at 14 the same circuit met such rows in its first passes and took 36.3 ms in place of 32.7.
 constexpr uint32_t kF64Spread = 20;
 constexpr int kF64MaxEntryExp = 60;                       // largest entry within 2^-60 .. 2^60
+// Entries are integers on the scale of the block's largest: one of 2^-k of it keeps 55 - k bits.  The
+// rotations by small angles of a Trotter step make entries of their own size on the way to rare
+// outcomes, so a block with an entry (that is not zero) below this runs on tile passes.
+constexpr double kF64MinEntry = 1.0 / (1 << 20);
 
 // A pass of one block over the state (a kernel parameter).  The tile: the block's 5 qubits
 // (columns c) and the 7 lowest others (rows m); 64 KiB in shared memory, element (m, c) at the
@@ -41,7 +45,8 @@ bool f64_pass_desc(int n, const int* q, F64Pass& P);
 // The B operand of a block, kF64B bytes, and its scale: the product of its gates, formed in
 // pairs of doubles (about 100 bits), so that one rounding per entry is left where the product
 // in double would round once per gate.  false if a sum of digit products that has to be exact
-// could exceed 2^24 (FP32 accumulation), or the largest entry is out of bounds (above) or not finite.
+// could exceed 2^24 (FP32 accumulation), or the largest entry is out of bounds (above) or not finite, or
+// another is too far below it.
 // matrix (32x32, row-major; may be null): the product rounded to FP64.
 bool f64_b_operand(const qs_gate* gates, const Block& b, unsigned char* out, int32_t* vs, cd* matrix = nullptr);
 

@@ -188,6 +188,12 @@ bool f64_b_operand(const qs_gate* gates, const Block& b, unsigned char* out, int
       big = std::max(big, std::max(std::abs(U.rh[r][c]), std::abs(U.ih[r][c])));
     }
   if (!(big > std::ldexp(1.0, -kF64MaxEntryExp) && big < std::ldexp(1.0, kF64MaxEntryExp))) return false;
+  // an entry far below the largest would keep few digits of its own (kF64MinEntry)
+  for (int r = 0; r < 32; ++r)
+    for (int c = 0; c < 32; ++c) {
+      const double a = std::max(std::abs(U.rh[r][c]), std::abs(U.ih[r][c]));
+      if (a != 0 && a < big * kF64MinEntry) return false;
+    }
   int e = 0;
   const double f = std::frexp(big, &e);   // big = f 2^e, 1/2 <= f < 1
   *vs = 55 - (f == 0.5 ? e - 1 : e);

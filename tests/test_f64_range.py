@@ -41,6 +41,11 @@ def scale_exe(tmp_path_factory):
     return _compile(tmp_path_factory, "f64_scale_check")
 
 
+@pytest.fixture(scope="module")
+def entry_exe(tmp_path_factory):
+    return _compile(tmp_path_factory, "f64_entry_check")
+
+
 def test_exponent_fields_of_accepted_blocks(scale_exe):
     # sizes over the range of doubles: a block that is taken keeps every result's exponent field in
     # 1 .. 2046, one that could not is refused
@@ -52,6 +57,51 @@ def test_exponent_fields_of_accepted_blocks(scale_exe):
     taken = [(int(lo), int(hi)) for _, ok, lo, hi in rows if ok == "1"]
     assert taken and all(1 <= lo and hi <= 2046 for lo, hi in taken)
     assert all(ok == "1" for s, ok, _, _ in rows if 2.0 ** -59 <= float(s) <= 2.0 ** 59)
+
+
+def test_entries_of_accepted_blocks_keep_their_digits(entry_exe):
+    # five rotations: entries from cos^5 down to sin^5.  An entry of 2^-k of the largest is held to 55 - k
+    # bits, and k <= 20 where the block is taken: half a unit of 2^-34 and as much for the reference's scale
+    angles = [1e-12, 1e-9, 1e-6, 1e-4, 1e-2, 0.05, 0.1, 0.13, 0.2, 0.5, 1.0, 1.5, 2.0, 3.0, 3.1, 3.1415]
+    r = subprocess.run([str(entry_exe), *map(str, angles)], capture_output=True, text=True, check=True)
+    rows = [x.split() for x in r.stdout.splitlines()]
+    for angle, (_, ok, err) in zip(angles, rows):
+        t = min(abs(np.tan(angle / 2)), 1 / abs(np.tan(angle / 2)))   # smallest entry over the largest: t^5
+        assert (ok == "1") == (t ** 5 >= 2.0 ** -20), angle
+        assert float(err) <= 2.0 ** -34, angle
+
+
+def _rotations_beside_dense(n, angle):
+    """RX by `angle` and CZ on qubits 0..4, Haar gates and CZs on the others."""
+    g = W.rng(23)
+    small, rest = [], []
+    for layer in range(3):
+        small += [("RX", (q,), (angle,), None) for q in range(5)]
+        small += [("CZ", (q, q + 1), (), None) for q in range(layer % 2, 4, 2)]
+    for layer in range(14):
+        rest += [("MAT1", (q,), (), W.haar_su2(g)) for q in range(5, n)]
+        rest += [("CZ", (q, q + 1), (), None) for q in range(5 + layer % 2, n - 1, 2)]
+    return small, rest
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("angle", [1e-6, 1e-3])
+def test_rare_outcomes_of_small_rotations(qs, angle):
+    # The state is a product: for every value of qubits 0..4 that of the others, times an amplitude of about
+    # angle^weight.  The rotations' block runs on tile passes (its entries reach down to angle^5), the others
+    # as blocks, with every amplitude to its own digits: 2^-34 of a row's amplitudes (kF64Spread) in each of
+    # about ten blocks, independent, four times that allowed
+    n = 16
+    small, rest = _rotations_beside_dense(n, angle)
+    st = qs.State(n, qs.QS_C128)
+    stats = qs.sv_apply_circuit(st, small + rest)
+    out = qs.sv_copy_out(st).reshape(-1, 32)
+    st.close()
+    assert 0 < stats["tile_launches"] < stats["passes"]
+    a = SV.apply_circuit(SV.basis(5), 5, small)
+    ref = SV.apply_circuit(SV.basis(n - 5), n - 5, [(k, tuple(q - 5 for q in qq), p, m) for k, qq, p, m in rest])
+    for j in range(32):
+        assert np.linalg.norm(out[:, j] / a[j] - ref) <= 4 * np.sqrt(10) * 2.0 ** -34, j
 
 
 @pytest.mark.gpu
