@@ -57,6 +57,19 @@ constexpr int kChainPart = 96 * 32 * 2;
 constexpr int kChainB = 3 * kChainPart;
 void chain_b_operand(const cd* U, unsigned char* out);
 
+// Which of the kernel's two pipelines takes block b of tile `step - b`.  Alternating over all blocks of all steps,
+// also those of tiles that are not there (before the first and after the last): a pipeline that takes
+// a tile's last block then takes that of one of the next two tiles, and never reaches a barrier whose phase
+// before last is still open.  (Counted over the items alone, the last tile of a pass of two blocks fell to the
+// pipeline of the first blocks, which did not know how far the stores were: with slow stores it passed
+// their barrier a phase early, wrote over a tile not yet stored and upset the count that the store waits for.)
+#ifdef __CUDACC__
+__host__ __device__
+#endif
+inline uint32_t chain_group(uint32_t step, int nblk, int b) {
+  return (step * (uint32_t)nblk + (uint32_t)b) & 1u;
+}
+
 // once per call, before its passes
 qs_status launch_chain_setup();
 qs_status launch_chain_pass(State* st, const ChainPass& P, const void* b_dev, int* status_dev);

@@ -21,7 +21,7 @@
 // the instructions and did not lower the error).
 //
 // Roles of the persistent CTA (one per SM; 20 warps), over items (tile t, block b).  Two equal
-// pipelines take alternate items, each with its own operand buffers, accumulator and warps:
+// pipelines take alternate items (chain_group), each with its own operand buffers, accumulator and warps:
 //   warps 0-3, 4-7    producers: thread = row = tensor-memory lane; read the row from the
 //                     tile's slot, split it, store the parts in tensor memory, a K half (16
 //                     columns) at a time
@@ -58,7 +58,8 @@ namespace {
 constexpr int kThreads = 640;
 constexpr int kSlotBytes = 4096 * 8;
 // Barriers of a kind are used in turn by the tiles (tile t: t mod kRing, use t / kRing),
-// whatever the number of slots, so that no role can meet a phase two uses away.
+// whatever the number of slots, and a role waits for a tile's only after it has passed one of the
+// kRing - 1 tiles before (chain_group), so that no role can meet a phase two uses away.
 constexpr uint32_t kRing = 4;
 constexpr int kWarpLoad = 16, kWarpStore = 18;   // 17 and 19 issue MMAs
 // tensor-memory columns: accumulator of pipeline g at 64 g (Re of the 32 outputs, then Im);
@@ -263,11 +264,10 @@ __global__ void __launch_bounds__(kThreads, 1)
     bool ok = true;
     for (uint32_t step = 0; step < steps && ok; ++step) {
       for (int b = 0; b < nblk && ok; ++b) {
-        if (step - (uint32_t)b >= my_tiles) continue;
-        const uint32_t it = item++;
-        if ((it & 1u) != grp) continue;
+        if (step - (uint32_t)b >= my_tiles || chain_group(step, nblk, b) != grp) continue;
+        const uint32_t it = item++;   // of this pipeline
         const uint32_t t = step - (uint32_t)b, ring = t % kRing, par = (t / kRing) & 1u;
-        const uint32_t buf = (it >> 1) & 1u, apar = (it >> 2) & 1u;
+        const uint32_t buf = it & 1u, apar = (it >> 1) & 1u;
         ok = warp_wait(b == 0 ? &full[ring] : &mfull[b - 1][ring], par, &s_fail);
         if (!ok) break;
         const uint32_t slot = b == 0 ? t % nload : nload + (uint32_t)b - 1u;
@@ -330,11 +330,10 @@ __global__ void __launch_bounds__(kThreads, 1)
     bool ok = true;
     for (uint32_t step = 0; step < steps && ok; ++step) {
       for (int b = 0; b < nblk && ok; ++b) {
-        if (step - (uint32_t)b >= my_tiles) continue;
-        const uint32_t it = item++;
-        if ((it & 1u) != grp) continue;
+        if (step - (uint32_t)b >= my_tiles || chain_group(step, nblk, b) != grp) continue;
+        const uint32_t it = item++;   // of this pipeline
         const uint32_t t = step - (uint32_t)b, ring = t % kRing;
-        ok = warp_wait(&dfull[grp], (it >> 1) & 1u, &s_fail);
+        ok = warp_wait(&dfull[grp], it & 1u, &s_fail);
         if (!ok) break;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         uint32_t re[32], im[32];
@@ -411,13 +410,12 @@ __global__ void __launch_bounds__(kThreads, 1)
     bool ok = true;
     for (uint32_t step = 0; step < steps && ok; ++step) {
       for (int b = 0; b < nblk && ok; ++b) {
-        if (step - (uint32_t)b >= my_tiles) continue;
-        const uint32_t it = item++;
-        if ((it & 1u) != grp) continue;
-        const uint32_t buf = (it >> 1) & 1u, apar = (it >> 2) & 1u;
+        if (step - (uint32_t)b >= my_tiles || chain_group(step, nblk, b) != grp) continue;
+        const uint32_t it = item++;   // of this pipeline
+        const uint32_t buf = it & 1u, apar = (it >> 1) & 1u;
         const uint64_t b0 = bdesc + (uint32_t)(b * (kChainB >> 4)), b1 = b0 + (256 >> 4);
         const uint32_t a0 = tm + kColA + 192u * grp + 96u * buf, a1 = a0 + kHalfCols;
-        ok = warp_wait(&dempty[grp], ((it >> 1) & 1u) ^ 1u, &s_fail) && warp_wait(&afull[grp][buf][0], apar, &s_fail);
+        ok = warp_wait(&dempty[grp], (it & 1u) ^ 1u, &s_fail) && warp_wait(&afull[grp][buf][0], apar, &s_fail);
         if (!ok) break;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         if (elect_one()) mma_corrections<true>(d, a0, b0, idesc);
