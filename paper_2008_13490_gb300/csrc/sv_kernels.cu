@@ -1726,19 +1726,18 @@ struct LogProduct {
   unsigned long long prod = 1ull << 63;   // the product's significand, prod / 2^63 in [1, 2)
   long long ex = 0;                       // and its exponent
   unsigned long long clamped = 0;
-  // p normal: its exponent; its significand times 2^31 (FP32) or 2^63
+  // p small(): its exponent; its significand times 2^31 (FP32) or 2^63
   __device__ __forceinline__ static int exponent(float p) { return (int)(__float_as_uint(p) >> 23) - 127; }
   __device__ __forceinline__ static int exponent(double p) { return (int)((uint32_t)__double2hiint(p) >> 20) - 1023; }
   __device__ __forceinline__ static uint32_t significand(float p) { return __float_as_uint(p) << 8 | 0x80000000u; }
   __device__ __forceinline__ static unsigned long long significand(double p) {
     return (unsigned long long)__double_as_longlong(p) << 11 | 1ull << 63;
   }
-  __device__ __forceinline__ static bool normal(float p) {
-    return (__float_as_uint(p) >> 23) - 1u < 254u;   // positive, neither subnormal nor infinite nor NaN
-  }
-  __device__ __forceinline__ static bool normal(double p) {
-    return ((uint32_t)__double2hiint(p) >> 20) - 1u < 2046u;
-  }
+  // Positive, not subnormal, and below 1/2.  An outcome from there on (one at most, of a distribution) takes
+  // its logarithm alone: near 1 that is far smaller than the parts of a sum of a significand's and an
+  // exponent's (of p = 1 - 1e-10 it had 34 bits).
+  __device__ __forceinline__ static bool small(float p) { return (__float_as_uint(p) >> 23) - 1u < 125u; }
+  __device__ __forceinline__ static bool small(double p) { return ((uint32_t)__double2hiint(p) >> 20) - 1u < 1021u; }
   // the upper 64 bits of prod * m: 2^62 or more
   __device__ __forceinline__ static unsigned long long high(unsigned long long a, uint32_t m) {
     return (a >> 32) * m + (((a & 0xffffffffull) * m) >> 32);
@@ -1749,7 +1748,7 @@ struct LogProduct {
   template <typename R>
   __device__ __forceinline__ void add(R p, uint32_t c) {
     if (c == 0) return;
-    if (c <= kMaxPower && normal(p)) {
+    if (c <= kMaxPower && small(p)) {
       const auto m = significand(p);
       int e = (int)c * (exponent(p) + 1);
       for (uint32_t k = 0; k < c; ++k) {
