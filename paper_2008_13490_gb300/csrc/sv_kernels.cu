@@ -1613,28 +1613,35 @@ __global__ void __launch_bounds__(256)
   if (threadIdx.x == 0) partials[blockIdx.x] = acc;
 }
 
-// A sum of FP32 numbers as an FP32 pair: every addition is split exactly into its rounded sum and
-// its remainder (Knuth), and only the sum of the remainders rounds, at 2^-24 of 2^-24 of the sum.
-// An FP64 addition holds its pipe for 64 cycles per warp, a conversion as long; these six
-// instructions take 6 issue slots.
+// A sum of FP32 numbers in three FP32 parts: an addition is split exactly into its rounded sum and its
+// remainder (Knuth), the remainders are added in the same way, and only the sum of their remainders rounds,
+// below FP64's unit.  (With the remainders summed plainly, 31 probabilities of 2^-25 beside one of 1 were off by
+// up to 2^-42.)  An FP64 addition per number instead: 1.14 ms for the marginals below.
 struct Sum32 {
-  float s = 0.f, e = 0.f;
+  float s = 0.f, e = 0.f, f = 0.f;
+  // a + b rounded; r: what that left out
+  __device__ __forceinline__ static float two_sum(float a, float b, float& r) {
+    const float t = a + b, v = t - a;
+    r = (a - (t - v)) + (b - v);
+    return t;
+  }
   __device__ __forceinline__ void add(float p) {
-    const float t = s + p, b = t - s;
-    e += (s - (t - b)) + (p - b);
-    s = t;
+    float r, q;
+    s = two_sum(s, p, r);
+    e = two_sum(e, r, q);
+    f += q;
   }
   __device__ __forceinline__ bool finite() const { return fabsf(s) <= 3.402823466e38f; }
-  __device__ __forceinline__ double value() const { return (double)s + (double)e; }
+  __device__ __forceinline__ double value() const { return (double)s + ((double)e + (double)f); }
 };
 
 // Marginal over the bits of a mask.  A warp reads lines of 32 amplitudes (address bits 0..4)
 // whose mask bits above are fixed, over a part of the remaining bits, so a lane's
-// probabilities all go to one outcome: they are summed in registers (FP32 states as pairs in
-// chunks, then FP64; a chunk that leaves FP32's range is summed again in FP64), across the lanes
+// probabilities all go to one outcome: they are summed in registers (FP32 states in three FP32
+// parts in chunks, then FP64; a chunk that leaves FP32's range is summed again in FP64), across the lanes
 // whose mask bits agree, and added to the outcome once.  HBM bounds it.  One shared-memory FP64
 // atomic per amplitude before: 28 qubits FP32, 10 low bits 1.86 ms, 10 high ones 18.9 ms; now
-// 0.46 and 0.45 ms (reading 2 GiB at the copy rate: 0.32 ms).
+// 0.62 ms (0.46 with sums of 45 bits; reading 2 GiB at the copy rate: 0.32 ms).
 struct MargPlan {
   uint8_t hi_pos[32];       // mask positions from 5 on, ascending
   int32_t n_hi, k_lo;       // of them; mask positions below 5
