@@ -369,7 +369,8 @@ __global__ void __launch_bounds__(kThreads, 1)
           const float* so = s_out[grp][k];
           const float ny = (so[0] + so[1]) + (so[2] + so[3]);
           const float diff = ((si[0] - so[0]) + (si[1] - so[1])) + ((si[2] - so[2]) + (si[3] - so[3]));
-          if (ny > 0.f) {
+          // (an infinity or a NaN stays with its row: the tile is then left as the products gave it)
+          if (ny > 0.f && fabsf(diff) <= 3.402823466e38f && ny <= 3.402823466e38f) {
             const float q = __fdividef(diff, ny);
             delta = fabsf(q) < 0x1p-10f ? q * fmaf(-0.125f, q, 0.5f)
                                         : diff / (ny + sqrtf(ny) * sqrtf((si[0] + si[1]) + (si[2] + si[3])));
