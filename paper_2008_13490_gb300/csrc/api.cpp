@@ -439,7 +439,8 @@ constexpr size_t kRunMin = 3;
 // the one at which they reach kMinScale, and the others become [1 1; 1 -1]: one addition per
 // amplitude, which rounds once, and no rounded constant in each.  (Ops are linear; no amplitude
 // grows by more than 1 / kMinScale in between.)  30-qubit Fourier transform: 46.1 -> 43.1 ms, error
-// against 64 bits 1.2e-6 -> 7.5e-7.
+// against 64 bits 1.2e-6 -> 7.5e-7.  Matrices of that shape whose factor is above 1 or far below it (explicit ones) are
+// left alone: their gathered factor could leave the range that the amplitudes keep.
 constexpr double kMinScale = 1.0 / 256;
 template <typename R>
 struct HadamardScale {
@@ -447,7 +448,7 @@ struct HadamardScale {
   TileOp<R>* last = nullptr;   // the latest Hadamard op, its factor in scale
   static bool is(const FOp& o) {
     const double h = o.type == F_G1 ? o.m0[0].real() : 0.0;
-    return h > 0 && o.m0[0] == cd(h) && o.m0[1] == cd(h) && o.m0[2] == cd(h) && o.m0[3] == cd(-h);
+    return h >= 0.5 && h <= 1 && o.m0[0] == cd(h) && o.m0[1] == cd(h) && o.m0[2] == cd(h) && o.m0[3] == cd(-h);
   }
   void add(const FOp& o, TileOp<R>* t) {
     if (!is(o)) return;
