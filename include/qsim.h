@@ -131,8 +131,10 @@ typedef enum {
    * block with an entry below 2^-20 of its largest runs on tile passes.  QS_METHOD_TILED
    * keeps FP64's relative precision of every amplitude.  Everything else uses
    * QS_METHOD_TILED.
-   * Synchronous like the block methods for complex64 states with n >= 12, and where
-   * complex128 blocks run. */
+   * Synchronous like the block methods for complex64 states with n >= 12.  A fault of the
+   * complex128 blocks' kernel (its bounded waits) is returned by the next call on the state that
+   * waits for its stream, or the next sv_apply_circuit.  On a stream that is being captured into a
+   * graph, complex128 states of n >= 12 run on tile passes. */
   QS_METHOD_AUTO = 4
 } qs_method;
 

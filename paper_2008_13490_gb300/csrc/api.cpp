@@ -78,6 +78,16 @@ qs_status ensure_opbuf(State* st, size_t bytes) {
   return QS_OK;
 }
 
+qs_status late_status(State* st) {
+  if (!st->late) return QS_OK;
+  const int code = *reinterpret_cast<volatile int*>(st->late);
+  if (code == 0) return QS_OK;
+  *st->late = 0;
+  set_error(code == QS_ETIMEOUT ? "complex128 block kernel: bounded wait gave up"
+                                : "complex128 block kernel: the tile slots do not fit shared memory");
+  return code == QS_ETIMEOUT ? QS_ETIMEOUT : QS_ECUDA;
+}
+
 // device buffer and pinned staging of at least `bytes`, the staging free to be written
 qs_status reserve_upload(State* st, size_t bytes) {
   qs_status s = ensure_opbuf(st, bytes);
@@ -1141,36 +1151,27 @@ qs_status run_blocks(State* st, const qs_gate* gates, size_t ngates, int mode, q
 }
 
 // One sweep per block over blocks [0, count), their operands (kF64Op bytes each) at `ops`, or null: then
-// they stand in the pinned buffer already, from byte 16 on.
+// they stand in the pinned buffer already.  Asynchronous: what the kernels report is taken by late_status.
 qs_status run_f64_list(State* st, const F64Pass* passes, size_t count, const unsigned char* ops, qs_stats* stats,
                        KernelTimer& tm) {
-  const size_t bytes = 16 + count * (size_t)kF64Op;   // status word, operands
+  const size_t bytes = count * (size_t)kF64Op;
   unsigned char* host = (unsigned char*)st->hostbuf;
   qs_status s = QS_OK;
   if (ops) {
     s = upload_begin(st, bytes, &host);
     if (s != QS_OK) return s;
-    std::memcpy(host + 16, ops, bytes - 16);
+    std::memcpy(host, ops, bytes);
   }
-  std::memset(host, 0, 16);
   unsigned char* dev = (unsigned char*)st->opbuf;
   s = upload_part(st, 0, bytes, true);
   for (size_t i = 0; i < count && s == QS_OK; ++i) {
     tm.before(4);
-    s = launch_f64_pass(st, passes[i], dev + 16 + i * kF64Op, (int*)dev);
+    s = launch_f64_pass(st, passes[i], dev + i * kF64Op, st->late);
     tm.after();
   }
   if (s != QS_OK) {
     cudaStreamSynchronize(st->stream);
     return s == QS_EUNSUPPORTED ? QS_ECUDA : s;
-  }
-  int status = 0;
-  QS_CUDA(cudaMemcpyAsync(&status, dev, sizeof(int), cudaMemcpyDeviceToHost, st->stream));
-  QS_CUDA(cudaStreamSynchronize(st->stream));
-  if (status != 0) {
-    set_error(status == QS_ETIMEOUT ? "complex128 block kernel: bounded wait gave up"
-                                    : "complex128 block kernel: the tile slots do not fit shared memory");
-    return status == QS_ETIMEOUT ? QS_ETIMEOUT : QS_ECUDA;
   }
   if (stats) {
     stats->ops_fused += (int64_t)count;
@@ -1228,10 +1229,18 @@ qs_status run_f64_blocks(State* st, const qs_gate* gates, size_t ngates, qs_stat
   for (size_t i = 0; i < nb; ++i)
     if (!f64_pass_desc(st->n, blocks[i].q, passes[i])) return QS_EUNSUPPORTED;
   unsigned char* host = nullptr;
-  qs_status s = upload_begin(st, 16 + nb * (size_t)kF64Op, &host);
+  qs_status s = upload_begin(st, nb * (size_t)kF64Op, &host);
   if (s != QS_OK) return s;
+  if (!st->late) {
+    if (cudaHostAlloc((void**)&st->late, sizeof(int), cudaHostAllocMapped) != cudaSuccess) {
+      cudaGetLastError();
+      st->late = nullptr;
+      return QS_EUNSUPPORTED;
+    }
+    *st->late = 0;
+  }
   parallel_for(nb, 2, [&](size_t i) {
-    unsigned char* const at = host + 16 + i * kF64Op;
+    unsigned char* const at = host + i * kF64Op;
     fits[i] = f64_b_operand(gates, blocks[i], at, &passes[i].vs, (cd*)(at + kF64B));
   });
   if (!mostly(fits)) return QS_EUNSUPPORTED;
@@ -1240,7 +1249,7 @@ qs_status run_f64_blocks(State* st, const qs_gate* gates, size_t ngates, qs_stat
   if (std::find(fits.begin(), fits.end(), (char)0) == fits.end())
     return run_f64_list(st, passes.data(), nb, nullptr, stats, tm);
   // (the tile passes' uploads take the pinned buffer)
-  const std::vector<unsigned char> ops(host + 16, host + 16 + nb * (size_t)kF64Op);
+  const std::vector<unsigned char> ops(host, host + nb * (size_t)kF64Op);
   for (size_t i = 0; i < nb && s == QS_OK;) {
     size_t j = i;
     while (j < nb && fits[j] == fits[i]) ++j;
@@ -1418,6 +1427,13 @@ qs_status adjoint_tiled(State* st, void* lam, const qs_gate* gates, size_t g0, s
 // (qs_stats.tile_launches).
 constexpr int kSmallAutoBits = 13;
 
+// Whether the state's stream is being captured into a graph.
+static bool capturing(const State* st) {
+  cudaStreamCaptureStatus c = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st->stream, &c) != cudaSuccess) cudaGetLastError();
+  return c != cudaStreamCaptureStatusNone;
+}
+
 qs_status apply_gates(State* st, const qs_gate* gates, size_t ngates, int method, qs_stats* stats,
                       int flags) {
   if (stats) std::memset(stats, 0, sizeof(*stats));
@@ -1427,9 +1443,13 @@ qs_status apply_gates(State* st, const qs_gate* gates, size_t ngates, int method
   }
   // AUTO: blocks and tile passes where the state allows the blocks, else tiles
   const bool autom = method == QS_METHOD_AUTO && st->prec == QS_C64 && st->n >= kTileBits;
-  const bool auto_small = method == QS_METHOD_AUTO && st->n <= kSmallAutoBits &&
+  const qs_status earlier = late_status(st);   // (of a call that has ended by now)
+  if (earlier != QS_OK) return earlier;
+  // (a captured complex128 call keeps to tile passes, whose launches hold all they need)
+  const bool captured = method == QS_METHOD_AUTO && st->prec == QS_C128 && st->n >= kTileBits && capturing(st);
+  const bool auto_small = method == QS_METHOD_AUTO && st->n <= kSmallAutoBits && !captured &&
                           (st->prec == QS_C128 || st->n < kSmallAutoBits || chains_likely(gates, ngates));
-  const bool auto_f64 = method == QS_METHOD_AUTO && st->prec == QS_C128 && st->n >= kTileBits && !auto_small;
+  const bool auto_f64 = method == QS_METHOD_AUTO && st->prec == QS_C128 && st->n >= kTileBits && !auto_small && !captured;
   if (method == QS_METHOD_AUTO && !autom) method = QS_METHOD_TILED;
   const bool blocks = method == QS_METHOD_BLOCKS_TF32 || method == QS_METHOD_BLOCKS_BF16;
   if (blocks && (st->prec != QS_C64 || st->n < kTileBits)) {
@@ -1465,6 +1485,7 @@ qs_status apply_gates(State* st, const qs_gate* gates, size_t ngates, int method
             : run_tiled<double>(st, fops, vmap, stats, tm);
   }
   tm.finish(stats);
+  if (tm.on && s == QS_OK) s = late_status(st);   // (the events have been waited for)
   if (stats) {
     stats->gates_in = (int64_t)ngates;
     stats->bytes_moved = (double)stats->passes * 2.0 * (double)st->data_bytes;
@@ -1690,6 +1711,7 @@ qs_status sv_destroy(qs_state_t st) {
     dev_free(st, st->scratch, st->scratch_bytes);
     if (st->owns_data) dev_free(st, st->data, st->data_bytes);
     if (st->hostbuf) cudaFreeHost(st->hostbuf);
+    if (st->late) cudaFreeHost(st->late);
     if (st->upload_done) cudaEventDestroy(st->upload_done);
     delete st;
     return QS_OK;
@@ -1702,7 +1724,7 @@ qs_status sv_set_stream(qs_state_t st, void* stream) {
     if (s != QS_OK) return s;
     QS_CUDA(cudaStreamSynchronize(st->stream));
     st->stream = (cudaStream_t)stream;
-    return QS_OK;
+    return late_status(st);
   });
 }
 
@@ -1760,6 +1782,7 @@ qs_status sv_copy_out(qs_state_t st, void* buf, int on_device) {
     } else {
       QS_CUDA(cudaMemcpyAsync(buf, st->data, st->data_bytes, cudaMemcpyDeviceToHost, st->stream));
       QS_CUDA(cudaStreamSynchronize(st->stream));
+      return late_status(st);
     }
     return QS_OK;
   });
@@ -1806,6 +1829,7 @@ qs_status sv_probs(qs_state_t st, void* out, int out_fp64, uint64_t marg_mask, d
       if (s != QS_OK) return s;
       QS_CUDA(cudaMemcpyAsync(norm_out, res, sizeof(double), cudaMemcpyDeviceToHost, st->stream));
       QS_CUDA(cudaStreamSynchronize(st->stream));
+      return late_status(st);
     }
     return QS_OK;
   });
@@ -1840,6 +1864,8 @@ qs_status sv_probs_host(qs_state_t st, void* host_out, int out_fp64, uint64_t ma
       QS_CUDA(cudaMemcpyAsync(h.data(), sc + kScratchMarg, h.size() * sizeof(double), cudaMemcpyDeviceToHost,
                               st->stream));
       QS_CUDA(cudaStreamSynchronize(st->stream));
+      s = late_status(st);
+      if (s != QS_OK) return s;
       if (out_fp64) std::memcpy(host_out, h.data(), h.size() * sizeof(double));
       else
         for (size_t i = 0; i < h.size(); ++i) ((float*)host_out)[i] = (float)h[i];
@@ -1857,7 +1883,7 @@ qs_status sv_probs_host(qs_state_t st, void* host_out, int out_fp64, uint64_t ma
         if (s == QS_OK && norm_out) s = sv_probs(st, nullptr, out_fp64, 0, norm_out);
         const cudaError_t e = cudaStreamSynchronize(st->stream);
         if (s == QS_OK && e != cudaSuccess) s = cuda_status(e, "sv_probs_host");
-        return s;
+        return s == QS_OK ? late_status(st) : s;
       }
       cudaGetLastError();   // a plain host pointer: not an error
     }
@@ -1884,7 +1910,7 @@ qs_status sv_probs_host(qs_state_t st, void* host_out, int out_fp64, uint64_t ma
     if (s == QS_OK && norm_out) s = sv_probs(st, nullptr, out_fp64, 0, norm_out);
     const cudaError_t e = cudaStreamSynchronize(st->stream);
     if (s == QS_OK && e != cudaSuccess) s = cuda_status(e, "sv_probs_host");
-    return s;
+    return s == QS_OK ? late_status(st) : s;
   });
 }
 
@@ -1922,7 +1948,8 @@ qs_status sv_probs_wait(qs_state_t st) {
   return abi_guard(__func__, [&]() -> qs_status {
     qs_status s = check_state(st);
     if (s != QS_OK) return s;
-    return wait_copies(st);
+    s = wait_copies(st);
+    return s == QS_OK ? late_status(st) : s;
   });
 }
 
@@ -1946,7 +1973,7 @@ qs_status sv_loglik(qs_state_t st, const uint32_t* counts, double* out, int64_t*
     QS_CUDA(cudaMemcpyAsync(&nc, sc + kScratchClamps, sizeof(nc), cudaMemcpyDeviceToHost, st->stream));
     QS_CUDA(cudaStreamSynchronize(st->stream));
     if (clamped) *clamped = (int64_t)nc;
-    return QS_OK;
+    return late_status(st);
   });
 }
 

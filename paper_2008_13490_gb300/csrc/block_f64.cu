@@ -191,7 +191,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   const uint32_t bsm = smem_u32(smem_raw);
   const uint32_t slots = (bsm + (uint32_t)kF64B + (kSlotBytes - 1u)) & ~(kSlotBytes - 1u);
   if (slots + 2u * kSlotBytes > bsm + (uint32_t)kDynSmem) {   // (the same for all threads)
-    if (tid == 0) atomicExch(status, (int)QS_EUNSUPPORTED);
+    if (tid == 0) *reinterpret_cast<volatile int*>(status) = (int)QS_EUNSUPPORTED;   // (host memory)
     return;
   }
   if (tid == 0) {
@@ -414,7 +414,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
-  if (tid == 0 && s_fail) atomicExch(status, (int)QS_ETIMEOUT);
+  if (tid == 0 && s_fail) *reinterpret_cast<volatile int*>(status) = (int)QS_ETIMEOUT;
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem) : "memory");
 }
 
@@ -456,7 +456,7 @@ qs_status launch_f64_setup() {
   return QS_OK;
 }
 
-qs_status launch_f64_pass(State* st, const F64Pass& P, const void* b_dev, int* status_dev) {
+qs_status launch_f64_pass(State* st, const F64Pass& P, const void* b_dev, int* status) {
   CUtensorMap map;
   const qs_status ms = f64_tensor_map(st, P, &map);
   if (ms != QS_OK) return ms;
@@ -467,7 +467,7 @@ qs_status launch_f64_pass(State* st, const F64Pass& P, const void* b_dev, int* s
   uint64_t grid = (uint64_t)std::max(1, sms - reserved_sms());   // (one CTA takes an SM's tensor memory)
   if (grid > ntiles) grid = ntiles;
   block_f64_kernel<<<(unsigned)grid, kThreads, kDynSmem, st->stream>>>(P, map, (const unsigned char*)b_dev,
-                                                                       (uint32_t)ntiles, status_dev);
+                                                                       (uint32_t)ntiles, status);
   QS_CUDA(cudaGetLastError());
   return QS_OK;
 }

@@ -51,7 +51,7 @@ bool f64_pass_desc(int n, const int* q, F64Pass& P);
 bool f64_b_operand(const qs_gate* gates, const Block& b, unsigned char* out, int32_t* vs, cd* matrix = nullptr);
 
 qs_status launch_f64_setup();
-// b_dev: kF64Op bytes
-qs_status launch_f64_pass(State* st, const F64Pass& P, const void* b_dev, int* status_dev);
+// b_dev: kF64Op bytes; status: page-locked host memory
+qs_status launch_f64_pass(State* st, const F64Pass& P, const void* b_dev, int* status);
 
 }  // namespace qs

@@ -73,7 +73,7 @@ qs_status device_checksum(State* st, uint64_t* sum) {
   QS_CUDA(cudaGetLastError());
   QS_CUDA(cudaMemcpyAsync(sum, d, sizeof(*sum), cudaMemcpyDeviceToHost, st->stream));
   QS_CUDA(cudaStreamSynchronize(st->stream));
-  return QS_OK;
+  return late_status(st);
 }
 
 struct Pinned {

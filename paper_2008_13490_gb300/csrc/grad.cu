@@ -427,7 +427,7 @@ qs_status run_grad(State* st, const qs_gate* gates, size_t ng, const double* w, 
   }
   dev_free(st, dth, 0);
   cleanup();
-  return s;
+  return s == QS_OK ? late_status(st) : s;
 }
 
 }  // namespace

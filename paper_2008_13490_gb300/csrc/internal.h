@@ -46,6 +46,9 @@ struct State {
   void* hostbuf = nullptr;
   size_t hostbuf_bytes = 0;
   cudaEvent_t upload_done = nullptr;
+  // status that a kernel of an asynchronous call leaves (page-locked, written by the device; null until
+  // such a call): taken by the next call that waits for the stream (late_status)
+  int* late = nullptr;
   // device staging buffer of probabilities bound for host memory (sv_probs_host)
   void* stage = nullptr;
   size_t stage_bytes = 0;
@@ -54,6 +57,9 @@ struct State {
 void* dev_alloc(State* st, size_t bytes);
 void dev_free(State* st, void* p, size_t bytes);
 qs_status ensure_opbuf(State* st, size_t bytes);
+// The status that kernels of earlier asynchronous calls left, which ends with this report.  To be called
+// when the state's stream has been waited for.
+qs_status late_status(State* st);
 
 // Per-state scratch (device): reduction partials, counters, small tables.
 constexpr int kReduceBlocks = 1024;               // partial sums written by reduction kernels

@@ -599,7 +599,7 @@ extern "C" qs_status sv_bloch(qs_state_t st_, double* r_out) {
     if (s != QS_OK) return s;
     QS_CUDA(cudaMemcpyAsync(r_out, dev_out, sizeof(double) * 3 * (size_t)n, cudaMemcpyDeviceToHost, st->stream));
     QS_CUDA(cudaStreamSynchronize(st->stream));
-    return QS_OK;
+    return late_status(st);
   });
 }
 

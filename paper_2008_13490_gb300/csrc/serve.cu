@@ -503,7 +503,7 @@ struct Server {
           if (s2 == QS_OK) {
             cudaError_t e = cudaMemcpyAsync(hbuf, marg, sizeof(double) << r->k, cudaMemcpyDeviceToHost, stream);
             if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
-            if (e != cudaSuccess) s2 = cuda_status(e, "large circuit readout");
+            s2 = e != cudaSuccess ? cuda_status(e, "large circuit readout") : late_status(st);
           }
           if (s2 == QS_OK) r->result.assign(hbuf, hbuf + ((size_t)1 << r->k));
           return s2;
