@@ -1214,6 +1214,7 @@ qs_status run_tile_segment(State* st, const qs_gate* gates, const std::vector<Bl
 // QS_EUNSUPPORTED, with nothing launched, for other circuits: they run on tile passes.
 qs_status run_f64_blocks(State* st, const qs_gate* gates, size_t ngates, qs_stats* stats, KernelTimer& tm) {
   if (!chains_likely(gates, ngates)) return QS_EUNSUPPORTED;
+  if (packed_ctas() > 0 && packed_ctas() != reserved_sms()) return QS_EUNSUPPORTED;   // (too few SMs free for a while)
   std::vector<Block> blocks;
   plan_blocks(gates, ngates, st->n, blocks, /*products=*/false);
   const size_t nb = blocks.size();
@@ -1405,7 +1406,7 @@ qs_status adjoint_small_t(State* st, void* lam, const qs_gate* gates, size_t ng,
 }
 
 qs_status adjoint_small(State* st, void* lam, const qs_gate* gates, size_t ng, double* dth) {
-  if (!gates_unitary(gates, ng)) return QS_EUNSUPPORTED;
+  if (!gates_unitary(gates, ng) || !small_fits(st)) return QS_EUNSUPPORTED;
   return st->prec == QS_C64 ? adjoint_small_t<float>(st, lam, gates, ng, dth)
                             : adjoint_small_t<double>(st, lam, gates, ng, dth);
 }
@@ -1448,6 +1449,7 @@ qs_status apply_gates(State* st, const qs_gate* gates, size_t ngates, int method
   // (a captured complex128 call keeps to tile passes, whose launches hold all they need)
   const bool captured = method == QS_METHOD_AUTO && st->prec == QS_C128 && st->n >= kTileBits && capturing(st);
   const bool auto_small = method == QS_METHOD_AUTO && st->n <= kSmallAutoBits && !captured &&
+                          (st->n < kTileBits || small_fits(st)) &&
                           (st->prec == QS_C128 || st->n < kSmallAutoBits || chains_likely(gates, ngates));
   const bool auto_f64 = method == QS_METHOD_AUTO && st->prec == QS_C128 && st->n >= kTileBits && !auto_small && !captured;
   if (method == QS_METHOD_AUTO && !autom) method = QS_METHOD_TILED;

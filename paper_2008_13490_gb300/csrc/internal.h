@@ -298,6 +298,10 @@ qs_status ptm_validate(const double* ptms, int n, int count, const char* what, i
 // SMs that block passes leave free while persistent packed kernels of servers
 // may run (serve.cu)
 int reserved_sms();
+// CTAs of persistent packed kernels that may be running (serve.cu)
+int packed_ctas();
+// Whether the small-state kernels' CTAs find SMs free beside those (sv_kernels.cu)
+bool small_fits(const State* st);
 
 // Applies gates to a state (the body of sv_apply_circuit; api.cpp).
 qs_status apply_gates(State* st, const qs_gate* gates, size_t ngates, int method, qs_stats* stats,
@@ -334,7 +338,7 @@ struct TermPar {
 qs_status launch_term_reduce(State* st, const void* partial, int nsum, const TermRec* recs, int nrec,
                              const TermPar* pars, double* dth);
 // The adjoint sweep of a state below a tile over gates [0, ng) in one launch; QS_EUNSUPPORTED
-// (nothing launched) when a matrix is not unitary.  Otherwise as adjoint_tiled.
+// (nothing launched) when a matrix is not unitary or a packed kernel leaves its cluster no room.  Otherwise as adjoint_tiled.
 qs_status adjoint_small(State* st, void* lam, const qs_gate* gates, size_t ng, double* dth);
 // PlainOps whose pad[0] is 1 + the op's first sum (0: none); partial: adjoint_small_warps x nsum
 int adjoint_small_warps(const State* st);

@@ -50,6 +50,9 @@ namespace qs {
 // SMs the block passes leave free for running persistent packed kernels
 std::atomic<int> g_reserved_sms{0};
 int reserved_sms() { return g_reserved_sms.load(); }
+// CTAs of running persistent packed kernels
+std::atomic<int> g_packed_ctas{0};
+int packed_ctas() { return g_packed_ctas.load(); }
 
 namespace {
 
@@ -244,7 +247,7 @@ struct Server {
   cudaStream_t pk_stream = nullptr;
   cudaEvent_t pk_ev = nullptr;
   bool pk_running = false;
-  int pk_reserved = 0;
+  int pk_ctas = 0, pk_reserved = 0;
   size_t pk_smem = 0, op_size = 0;
   PCtl* ctl = nullptr;               // mapped host memory from here ...
   PJob* jobs = nullptr;
@@ -390,11 +393,19 @@ struct Server {
     return any;
   }
 
+  // what the packed kernel holds while it runs: `ctas` CTAs, 0 once it has ended
+  void hold_sms(int ctas) {
+    const int reserve = std::min(ctas, sms / 2);
+    g_packed_ctas.fetch_add(ctas - pk_ctas);
+    g_reserved_sms.fetch_add(reserve - pk_reserved);
+    pk_ctas = ctas;
+    pk_reserved = reserve;
+  }
+
   qs_status launch_persistent() {
     QS_CUDA(cudaMemsetAsync(d_status, 0, sizeof(int), pk_stream));
     const int P = cfg.persistent_ctas;
-    pk_reserved = std::min(P, sms / 2);
-    g_reserved_sms.fetch_add(pk_reserved);
+    hold_sms(P);
     const uint64_t idle_ns = (uint64_t)cfg.idle_ms * 1000000ull;
     if (cfg.prec == QS_C64)
       packed_persistent_kernel<float><<<P, 256, pk_smem, pk_stream>>>(
@@ -407,8 +418,7 @@ struct Server {
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaEventRecord(pk_ev, pk_stream);
     if (e != cudaSuccess) {
-      g_reserved_sms.fetch_sub(pk_reserved);
-      pk_reserved = 0;
+      hold_sms(0);
       return cuda_status(e, "persistent packed kernel launch");
     }
     pk_running = true;
@@ -453,14 +463,12 @@ struct Server {
       cudaStreamSynchronize(pk_stream);   // nothing of it may still run when the queue starts over
       cudaGetLastError();
       pk_running = false;
-      g_reserved_sms.fetch_sub(pk_reserved);
-      pk_reserved = 0;
+      hold_sms(0);
       fail_queue(st, msg);
       return true;
     }
     pk_running = false;
-    g_reserved_sms.fetch_sub(pk_reserved);
-    pk_reserved = 0;
+    hold_sms(0);
     int status = 0;
     if (cudaMemcpy(&status, d_status, sizeof(int), cudaMemcpyDeviceToHost) == cudaSuccess &&
         status == (int)QS_ETIMEOUT) {
@@ -805,7 +813,7 @@ qs_status qs_server_destroy(qs_server_t s) {
       if (w.joinable()) w.join();
     if (s->ctl) reinterpret_cast<std::atomic<uint32_t>*>(&s->ctl->stop)->store(1u, std::memory_order_release);
     if (s->pk_stream) cudaStreamSynchronize(s->pk_stream);   // the kernel ends at its next wait
-    if (s->pk_reserved) g_reserved_sms.fetch_sub(s->pk_reserved);
+    s->hold_sms(0);
     for (auto& kv : s->reqs) delete kv.second;
     if (s->pk_stream) cudaStreamDestroy(s->pk_stream);
     if (s->pk_ev) cudaEventDestroy(s->pk_ev);

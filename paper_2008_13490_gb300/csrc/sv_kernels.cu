@@ -1258,6 +1258,19 @@ __global__ void __launch_bounds__(1024)
   if (clustered) cluster_barrier();                               // nobody reads this CTA's buffers any more
 }
 
+// The same for a state below a tile on one CTA of 256 threads that finds room on an SM beside a CTA of the
+// packed kernel: amplitudes in shared memory, an op at a time (the code of that kernel).
+template <typename R>
+__global__ void __launch_bounds__(256)
+    small_shared_kernel(C2<R>* __restrict__ psi, int n, const PlainOp<R>* __restrict__ ops, int nops) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  C2<R>* sm = reinterpret_cast<C2<R>*>(smem_raw);
+  for (int J = threadIdx.x; J < 1 << n; J += blockDim.x) sm[J] = psi[J];
+  __syncthreads();
+  small_apply_ops(sm, n, ops, nops);
+  for (int J = threadIdx.x; J < 1 << n; J += blockDim.x) psi[J] = sm[J];
+}
+
 // The adjoint sweep of a small state: psi and lambda as in small_state_kernel, an amplitude of each
 // per thread, through the ops of a run list (PlainOp::pad[0] = 1 + the index of the op's first sum,
 // 0: none).  A warp's sums go to partial[warp][sum], in the state's precision within a warp and FP64
@@ -2010,6 +2023,42 @@ static qs_status small_launch_t(State* st, const void* ops_dev, int nops) {
                       (const PlainOp<R>*)ops_dev, nops);
 }
 
+// A cluster waits until as many SMs of one GPC are free as it has CTAs: beside a persistent packed kernel
+// (a CTA on each SM it holds, whatever is left there too little for one of 1024 threads) that can last
+// until the kernel's end.  It certainly fits while the packed CTAs are fewer than the clusters that fit an empty
+// device, one CTA to an SM, or leave more SMs than (cluster - 1) for each of these: some GPC then has
+// `cluster` free.  (Every GPC holds a cluster of 8 here; 152 SMs in GPCs of 16 to 20.)
+bool small_fits(const State* st) {
+  const int held = packed_ctas();
+  if (held == 0) return true;
+  const int cluster = 1 << (st->n - small_tbits(st));
+  int dev = 0, sms = 152, most = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (cluster == 1) return held < sms;
+  constexpr size_t kWhole = 160 * 1024;   // shared memory that two CTAs cannot have on an SM
+  auto clusters = [&](auto kernel) {
+    if (set_smem(kernel, kWhole) != QS_OK) return;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(cluster);
+    cfg.blockDim = dim3(1u << std::max(small_tbits(st), 5));
+    cfg.dynamicSmemBytes = kWhole;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = cluster;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    if (cudaOccupancyMaxActiveClusters(&most, kernel, &cfg) != cudaSuccess) {
+      cudaGetLastError();
+      most = 0;
+    }
+  };
+  if (st->prec == QS_C64) clusters(&small_state_kernel<float>);
+  else clusters(&small_state_kernel<double>);
+  return held < std::max(most, sms - most * (cluster - 1));
+}
+
 int adjoint_small_warps(const State* st) {
   const int tbits = small_tbits(st);
   return (1 << (st->n - tbits)) * (1 << (std::max(tbits, 5) - 5));
@@ -2034,7 +2083,19 @@ qs_status launch_adjoint_small(State* st, void* lam, const void* ops_dev, int no
   return QS_OK;
 }
 
+template <typename R>
+static qs_status small_shared_launch_t(State* st, const void* ops_dev, int nops) {
+  const size_t smem = sizeof(C2<R>) << st->n;
+  qs_status s = set_smem(small_shared_kernel<R>, smem);
+  if (s != QS_OK) return s;
+  small_shared_kernel<R><<<1, 256, smem, st->stream>>>((C2<R>*)st->data, st->n, (const PlainOp<R>*)ops_dev, nops);
+  QS_CUDA(cudaGetLastError());
+  return QS_OK;
+}
+
 qs_status launch_small(State* st, const void* ops_dev, int nops) {
+  if (!small_fits(st))
+    return st->prec == QS_C64 ? small_shared_launch_t<float>(st, ops_dev, nops) : small_shared_launch_t<double>(st, ops_dev, nops);
   return st->prec == QS_C64 ? small_launch_t<float>(st, ops_dev, nops) : small_launch_t<double>(st, ops_dev, nops);
 }
 
