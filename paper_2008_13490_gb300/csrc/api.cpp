@@ -1231,6 +1231,7 @@ qs_status run_f64_blocks(State* st, const qs_gate* gates, size_t ngates, qs_stat
     if (!f64_pass_desc(st->n, blocks[i].q, passes[i])) return QS_EUNSUPPORTED;
   unsigned char* host = nullptr;
   qs_status s = upload_begin(st, nb * (size_t)kF64Op, &host);
+  if (s == QS_ENOMEM) return QS_EUNSUPPORTED;   // (tile passes need less)
   if (s != QS_OK) return s;
   if (!st->late) {
     if (cudaHostAlloc((void**)&st->late, sizeof(int), cudaHostAllocMapped) != cudaSuccess) {
@@ -1385,15 +1386,13 @@ qs_status adjoint_small_t(State* st, void* lam, const qs_gate* gates, size_t ng,
   }
   const size_t pbytes = sizeof(double) * (size_t)adjoint_small_warps(st) * kSums;
   double* partial = (double*)dev_alloc(st, pbytes);
-  if (!partial) {
-    set_error("adjoint partials allocation failed");
-    return QS_ENOMEM;
-  }
+  if (!partial) return QS_EUNSUPPORTED;   // (gate by gate takes less)
   std::vector<unsigned char> blob;
   const size_t off_ops = put(blob, ops.data(), ops.size());
   const size_t off_recs = put(blob, recs.data(), recs.size());
   const size_t off_pars = put(blob, ad.pars.data(), ad.pars.size());
   s = upload(st, blob);
+  if (s == QS_ENOMEM) s = QS_EUNSUPPORTED;   // (nothing launched)
   unsigned char* dev = (unsigned char*)st->opbuf;
   for (size_t i = 0; i < parts.size() && s == QS_OK; ++i) {
     const Part& q = parts[i];
@@ -1479,6 +1478,10 @@ qs_status apply_gates(State* st, const qs_gate* gates, size_t ngates, int method
     build_fused_ops(gates, ngates, st->n, fops, vmap, /*fuse=*/true, /*relabel=*/false);
     merge_one_qubit_ops(fops, st->n, nullptr);   // one CTA runs them all: no passes to keep
     s = c64 ? run_small<float>(st, fops, stats, tm) : run_small<double>(st, fops, stats, tm);
+    if (s == QS_ENOMEM && st->n >= kTileBits) {   // (all of its ops at once on the device; tile passes carry theirs along)
+      build_fused_ops(gates, ngates, st->n, fops, vmap, /*fuse=*/true, /*relabel=*/true);
+      s = c64 ? run_tiled<float>(st, fops, vmap, stats, tm) : run_tiled<double>(st, fops, vmap, stats, tm);
+    }
     // (the default method of complex64 states from kTileBits on returns when the state is ready)
     if (autom && s == QS_OK) QS_CUDA(cudaStreamSynchronize(st->stream));
   } else {

@@ -338,7 +338,8 @@ struct TermPar {
 qs_status launch_term_reduce(State* st, const void* partial, int nsum, const TermRec* recs, int nrec,
                              const TermPar* pars, double* dth);
 // The adjoint sweep of a state below a tile over gates [0, ng) in one launch; QS_EUNSUPPORTED
-// (nothing launched) when a matrix is not unitary or a packed kernel leaves its cluster no room.  Otherwise as adjoint_tiled.
+// (nothing launched) when a matrix is not unitary, a packed kernel leaves its cluster no room, or its
+// buffers cannot be had.  Otherwise as adjoint_tiled.
 qs_status adjoint_small(State* st, void* lam, const qs_gate* gates, size_t ng, double* dth);
 // PlainOps whose pad[0] is 1 + the op's first sum (0: none); partial: adjoint_small_warps x nsum
 int adjoint_small_warps(const State* st);
