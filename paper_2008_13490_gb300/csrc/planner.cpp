@@ -269,11 +269,12 @@ void build_fused_ops(const qs_gate* gates, size_t ngates, int n, std::vector<FOp
     }
     // In a tile pass (relabel) a real op (H, RY, X, CNOT) takes half the instructions of a complex one,
     // and a phase that meets another on the op's qubit is an entry of their run, which costs less than
-    // the op's becoming complex; a lone phase would be an op of its own, and is folded.  Kernels of a
-    // pass list, us, all folded / none into real ops / by this rule: Fourier transform of 25 qubits
-    // complex64 1317 / 1111 / 1120, of 22 complex128 2506 / 1645 / 1700; Hadamards with 1.5 phases each
-    // between random qubits, 25 qubits complex64 2051 / 1718 / 1734; layers of RY and neighbouring CP,
-    // 25 qubits complex64 4088 / 6718 / 4088, 22 complex128 14382 / 20298 / 14379.
+    // the op's becoming complex; one lone phase on either side would be an op of its own, and is folded.
+    // Kernels of a pass list, us, all folded / none into real ops / by this rule: Fourier transform of 25
+    // qubits complex64 1317 / 1111 / 1105, of 22 complex128 2506 / 1645 / 1642; Hadamards with 1.5 phases each
+    // between random qubits, 25 qubits complex64 2051 / 1718 / 1668, 22 complex128 5799 / 3618 / 3772; layers of RY
+    // and neighbouring CP, 25 qubits complex64 4088 / 6718 / 4075, 22 complex128 14382 / 20298 / 14375.  (A
+    // real op's products round less, too: the Fourier transforms' error is that of none folded.)
     // Lists for one CTA (small states, the server) have no real path: there all is folded (10 layers of
     // RY and CP on 10 qubits: 59 ops, 137 with the phases left).
     std::vector<std::vector<int>> phases(relabel ? n : 0);   // per qubit, in each gap between its ops
@@ -285,9 +286,12 @@ void build_fused_ops(const qs_gate* gates, size_t ngates, int n, std::vector<FOp
         if (is_phase(out[i]))
           for (int q : {out[i].a, out[i].b}) ++phases[q][gap(q, i)];
     }
-    auto stays_real = [&](const FOp& D, size_t i, const FOp& G) {
-      return relabel && (G.type == F_G1 || G.type == F_G1C) && (G.t == D.a || G.t == D.b) && is_phase(D) &&
-             is_real(G) && phases[G.t][gap(G.t, i)] >= 2;
+    auto stays_real = [&](const FOp& D, size_t g) {   // D beside op g: the phases on both sides of it
+      const FOp& G = out[g];
+      if (!relabel || (G.type != F_G1 && G.type != F_G1C) || (G.t != D.a && G.t != D.b) || !is_phase(D) || !is_real(G))
+        return false;
+      const size_t after = gap(G.t, g);   // (upper bound: past g itself)
+      return phases[G.t][after - 1] + phases[G.t][after] >= 3;
     };
     for (size_t i = 0; i < out.size(); ++i) {
       if (out[i].type != F_D) continue;
@@ -303,8 +307,8 @@ void build_fused_ops(const qs_gate* gates, size_t ngates, int n, std::vector<FOp
         auto jt = std::lower_bound(L.begin(), L.end(), (int)i);
         if (jt != L.begin() && *(jt - 1) > before) before = *(jt - 1);
       }
-      bool done = after >= 0 && !stays_real(D, i, out[(size_t)after]) && fold_into(D, out[(size_t)after], /*after=*/false);
-      if (!done && before >= 0 && !stays_real(D, i, out[(size_t)before]))
+      bool done = after >= 0 && !stays_real(D, (size_t)after) && fold_into(D, out[(size_t)after], /*after=*/false);
+      if (!done && before >= 0 && !stays_real(D, (size_t)before))
         done = fold_into(D, out[(size_t)before], /*after=*/true);
       if (done) dead[i] = 1;
     }
