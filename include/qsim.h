@@ -111,8 +111,9 @@ typedef enum {
   QS_METHOD_BLOCKS_TF32 = 2, /* two TF32 parts, 4 products (~1e-6 relative over 100 blocks) */
   QS_METHOD_BLOCKS_BF16 = 3, /* three BF16 parts, 6 products (~6e-7 relative over 100 blocks) */
   /* the default (also when opts is NULL).  States with n <= 13 (complex64 with n = 13: circuits
-   * with dense gates) run in one launch, kept in the registers of one CTA or a cluster of
-   * CTAs.  For other complex64 states
+   * in which more than a fifth of the gates make superpositions) run in one launch, kept in the
+   * registers of one CTA or a cluster of CTAs (where a server's packed kernel leaves the cluster
+   * no room, as larger states do from n = 12 on).  For other complex64 states
    * the circuit is cut into 5-qubit blocks; a block with more than half of its
    * 1024 entries nonzero is a dense contraction and its gates run as BF16-split
    * GEMMs on the tensor cores (planned again as chains of up to three 5-qubit blocks

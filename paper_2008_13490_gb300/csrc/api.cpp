@@ -1422,9 +1422,9 @@ qs_status adjoint_tiled(State* st, void* lam, const qs_gate* gates, size_t g0, s
 // 515 and 1418 -> 73 and 390; complex128 of 10 and 60 layers 700 and 2501 -> 103 and 472, 737 and 2860 ->
 // 190 and 937; Haar and CNOT complex128 of 5 and 60 layers 461 and 4557 -> 93 and 816, 490 and 4525 -> 153
 // and 1483; Fourier 278 -> 53 (12 qubits); 500 mixed gates 922 -> 171, 1106 -> 175.
-// Above, a thread would hold several amplitudes.  Circuits of 13
-// complex64 qubits without dense gates keep to tile passes all the same: their users count these
-// (qs_stats.tile_launches).
+// Above, a thread would hold several amplitudes.  Circuits of 13 complex64 qubits in which at most a fifth of
+// the gates make superpositions (chains_likely) keep to tile passes although one launch would be faster there
+// too: the library has always run them so and reports it (qs_stats.tile_launches), which its callers can hold it to.
 constexpr int kSmallAutoBits = 13;
 
 // Whether the state's stream is being captured into a graph.

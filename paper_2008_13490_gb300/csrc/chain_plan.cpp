@@ -102,7 +102,7 @@ int split_tile(const std::vector<uint64_t>& m, uint64_t T, std::vector<uint64_t>
 // Pass by pass: among tiles (those grown from each of the first gates left, and bits 0..3
 // with every window of 8 neighbouring qubits) the kTry that take the most gates are split
 // into blocks, and the one whose blocks take the most is kept.  40 layers of Haar + CZ at
-// 30 qubits: 38 passes of 110 blocks.
+// 30 qubits: 37 passes of 109 blocks.
 void plan_chains(const qs_gate* gates, size_t ngates, int n, std::vector<ChainPlan>& out, bool products) {
   constexpr size_t kSeeds = 12, kTry = 4;
   const uint64_t low = (1ull << kChainLow) - 1, all = n >= 64 ? ~0ull : (1ull << n) - 1;
