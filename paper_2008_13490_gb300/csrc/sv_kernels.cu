@@ -1654,7 +1654,7 @@ struct Sum32 {
 // parts in chunks, then FP64; a chunk that leaves FP32's range is summed again in FP64), across the lanes
 // whose mask bits agree, and added to the outcome once.  HBM bounds it.  One shared-memory FP64
 // atomic per amplitude before: 28 qubits FP32, 10 low bits 1.86 ms, 10 high ones 18.9 ms; now
-// 0.62 ms (0.46 with sums of 45 bits; reading 2 GiB at the copy rate: 0.32 ms).
+// 0.40 ms (0.61 when a batch was loaded after the last had been summed; reading 2 GiB at the copy rate: 0.32 ms).
 struct MargPlan {
   uint8_t hi_pos[32];       // mask positions from 5 on, ascending
   int32_t n_hi, k_lo;       // of them; mask positions below 5
@@ -1690,14 +1690,20 @@ __global__ void __launch_bounds__(256)
       const int cnt = (int)(lines - r0 < (uint64_t)kChunk ? lines - r0 : (uint64_t)kChunk);
       const uint64_t a0 = a;
       Sum32 k;
-      for (int rb = 0; rb < cnt; rb += kBatch) {   // cnt: a power of two
-        C2<R> v[kBatch];
+      C2<R> v[kBatch], nx[kBatch];   // a batch, and the next one on its way
+      auto fetch = [&](int rb) {
 #pragma unroll
         for (int r = 0; r < kBatch; ++r) {
-          v[r].x = v[r].y = R(0);
-          if (live && rb + r < cnt) v[r] = psi[(fixed | a) + lane];
+          nx[r].x = nx[r].y = R(0);
+          if (live && rb + r < cnt) nx[r] = psi[(fixed | a) + lane];
           a = ((a | ~P.rest) + 1) & P.rest;   // the next line
         }
+      };
+      fetch(0);
+      for (int rb = 0; rb < cnt; rb += kBatch) {   // cnt: a power of two
+#pragma unroll
+        for (int r = 0; r < kBatch; ++r) v[r] = nx[r];
+        if (rb + kBatch < cnt) fetch(rb + kBatch);
 #pragma unroll
         for (int r = 0; r < kBatch; ++r) {
           const R p = v[r].x * v[r].x + v[r].y * v[r].y;
