@@ -1224,8 +1224,11 @@ qs_status run_f64_blocks(State* st, const qs_gate* gates, size_t ngates, qs_stat
     for (size_t i = 0; i < nb; ++i) dense += is_dense[i] && also[i];
     return dense > 0 && dense >= 3 * (nb - dense);
   };
-  for (size_t i = 0; i < nb; ++i) is_dense[i] = block_dense(gates, blocks[i]);
-  if (!mostly(is_dense)) return QS_EUNSUPPORTED;
+  for (size_t i = 0, sparse = 0; i < nb; ++i) {
+    is_dense[i] = block_dense(gates, blocks[i]);
+    sparse += !is_dense[i];
+    if (4 * sparse > nb) return QS_EUNSUPPORTED;   // (decided: the rest need not be looked at)
+  }
   std::vector<F64Pass> passes(nb);
   for (size_t i = 0; i < nb; ++i)
     if (!f64_pass_desc(st->n, blocks[i].q, passes[i])) return QS_EUNSUPPORTED;

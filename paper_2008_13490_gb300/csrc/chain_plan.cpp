@@ -227,10 +227,15 @@ bool chains_likely(const qs_gate* gates, size_t ngates) {
 }
 
 bool chains_dense(const qs_gate* gates, const std::vector<ChainPlan>& plan) {
-  int dense = 0, sparse = 0;
+  size_t total = 0, dense = 0, sparse = 0;
+  for (const ChainPlan& p : plan) total += p.blocks.size();
   for (const ChainPlan& p : plan)
-    for (const Block& b : p.blocks) ++(block_dense(gates, b) ? dense : sparse);
-  return dense > 0 && dense >= 3 * sparse;
+    for (const Block& b : p.blocks) {
+      ++(block_dense(gates, b) ? dense : sparse);
+      if (4 * dense >= 3 * total) return true;   // (decided: the rest need not be looked at)
+      if (4 * sparse > total) return false;
+    }
+  return false;
 }
 
 namespace {
